@@ -129,6 +129,20 @@ cudaError_t jacobian_apply(int N, double h, const double *t, const double *v, do
 cudaError_t linear_sweep(int N, double h, float *e, const float *f, const float *th, int sweeps,
                          float *work, cudaStream_t s);
 
+// ---- the small levels of a V-cycle in one launch (recon_tail.cu)
+cudaError_t prepare_tails();
+// whether a tail may start on a level of side N
+template <typename T>
+bool tail_ok(int N);
+// the FAS V-cycle from level l down on t, g.  raw: g is the restricted
+// residual of the level above; the right side is formed from it first and the
+// level's scale factor is left in its scalar slots
+template <typename T>
+cudaError_t fas_tail(recon_handle *H, int l, T *t, const T *g, const double *cptr, bool raw);
+// the linear V-cycle from level l down on e32, f32 (levels with stored
+// cofactors).  raw: f's mean is removed first; zero: e starts from 0
+cudaError_t lin_tail(recon_handle *H, int l, bool raw, bool zero);
+
 // ---- the solvers (recon_mg.cu)
 recon_status solve_f64(recon_handle *H, const double *b, double *phi, double tol,
                        int max_cycles, recon_stats *st);

@@ -197,57 +197,6 @@ __device__ __forceinline__ Nb19<float> gather_at(int pm, int pc, int pp, int S, 
     return v;
 }
 
-// Eq. update for two cells, written on A = I + H theta directly.  With
-// s = tr A and the diagonal cofactors' sum S = tr adj A, the cell cubic is
-// f(s) = 27 (det A - rhs) with f'(s) = 9 S, so Newton's step on the cubic
-// (eq. update's root by one Newton step) is
-//     tau = (det A - rhs) / S,   theta_c += (h^2 / 2) tau
-// (every diagonal entry of A moves by -tau).  It is kept from the right of
-// the cubic's local minimum (s > 0, S > 0) when |f| does not grow, which for
-// the cubic is |tau| |s - tau| <= S (f(s + d) = d^2 (3 s + d) at the Newton
-// step d = -3 tau), evaluated without cancellation.  Otherwise the paper's
-// update (the largest root, Newton-polished) with p = 9 S - 3 s^2 and
-// q = 27 det A - 9 s S + 2 s^3 - 27 rhs; that rare fallback runs behind one
-// warp vote, so the common path has no divergent branch.  Call with all lanes.
-__device__ __forceinline__ float2 fas_update2_det(const Nb19<float2> &n, float2 rhs, float ih2, float h2_2,
-                                                  float h2_6, int rule)
-{
-    const float2 axx = fma2(fma2(n.c, f2(-2.0f), add2(n.xp, n.xm)), f2(ih2), f2(1.0f));
-    const float2 ayy = fma2(fma2(n.c, f2(-2.0f), add2(n.yp, n.ym)), f2(ih2), f2(1.0f));
-    const float2 azz = fma2(fma2(n.c, f2(-2.0f), add2(n.zp, n.zm)), f2(ih2), f2(1.0f));
-    const float2 q4 = f2(0.25f * ih2);
-    const float2 hxy = mul2(edge2(n.xpyp, n.xmym, n.xmyp, n.xpym), q4);
-    const float2 hyz = mul2(edge2(n.ypzp, n.ymzm, n.ymzp, n.ypzm), q4);
-    const float2 hxz = mul2(edge2(n.xpzp, n.xmzm, n.xmzp, n.xpzm), q4);
-    const float2 cxx = fma2(hyz, neg2(hyz), mul2(ayy, azz));
-    const float2 cyy = fma2(hxz, neg2(hxz), mul2(axx, azz));
-    const float2 czz = fma2(hxy, neg2(hxy), mul2(axx, ayy));
-    const float2 cxy = fma2(hxz, hyz, neg2(mul2(hxy, azz)));
-    const float2 cxz = fma2(hxy, hyz, neg2(mul2(hxz, ayy)));
-    const float2 det = fma2(axx, cxx, fma2(hxy, cxy, mul2(hxz, cxz)));
-    const float2 S = add2(add2(cxx, cyy), czz);
-    const float2 s = add2(add2(axx, ayy), azz);
-    const float2 F = sub2(det, rhs);
-    const float2 tau = mul2(F, rcp2(S));
-    const float2 u = mul2(tau, sub2(s, tau));
-    float2 out = fma2(tau, f2(h2_2), n.c);
-    const bool okx = rule == 0 && s.x > 0.0f && S.x > 0.0f && fabsf(u.x) <= S.x;
-    const bool oky = rule == 0 && s.y > 0.0f && S.y > 0.0f && fabsf(u.y) <= S.y;
-    if (!__all_sync(0xffffffffu, okx && oky)) {
-        if (!okx) {
-            const float p = 9.0f * S.x - 3.0f * s.x * s.x;
-            const float q = 27.0f * (det.x - rhs.x) + s.x * (2.0f * s.x * s.x - 9.0f * S.x);
-            out.x = n.c.x - h2_6 * (root_polished_ool(p, q) - s.x);
-        }
-        if (!oky) {
-            const float p = 9.0f * S.y - 3.0f * s.y * s.y;
-            const float q = 27.0f * (det.y - rhs.y) + s.y * (2.0f * s.y * s.y - 9.0f * S.y);
-            out.y = n.c.y - h2_6 * (root_polished_ool(p, q) - s.y);
-        }
-    }
-    return out;
-}
-
 // OLD-plane offset of the tile cell (jl, kl), jl in [-2, kBJ + 1], kl in [-2, kBK + 1]
 __device__ __forceinline__ int opos(int jl, int kl) { return (jl + 2) * kHOR + (kl & 1) * kHOH + ((kl + 2) >> 1); }
 
