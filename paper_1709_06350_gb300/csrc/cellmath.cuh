@@ -170,54 +170,91 @@ __device__ __forceinline__ T root_polished(T p, T q)
     return sn;
 }
 
-// right of the cubic's local minimum: s > sqrt(-p/3).  FP32 tests the
-// equivalent s > 0 and 3 s^2 > -p (no square root); FP64 keeps the
-// square root of the definition.
-__device__ __forceinline__ bool right_of_min(double s, double p)
-{
-    return s > m_sqrt(p < 0.0 ? -p * (1.0 / 3.0) : 0.0);
-}
-__device__ __forceinline__ bool right_of_min(float s, float p) { return s > 0.0f && 3.0f * s * s > -p; }
-
-// the Newton quotient f / f': IEEE in FP64, the fast reciprocal form
-// (2 ulp) in the FP32 smoother, whose result the defect correction refines
-__device__ __forceinline__ double newton_quot(double f, double fp) { return f / fp; }
-__device__ __forceinline__ float newton_quot(float f, float fp) { return __fdividef(f, fp); }
-
-// keep the Newton step s_new = s - quot (quot = f / f') if |f(s_new)| <= |f(s)|.
-// FP64 evaluates f(s_new).  FP32 uses the same test in the cancellation-free
-// form: f(s + d) = f + f' d + 3 s d^2 + d^3 = d^2 (3 s + d) for d = -quot, so
-// the test is |d| |3 s + d| <= f'; recomputing f(s_new) in FP32 near
-// convergence gives rounding noise, which rejected good steps at random.
-__device__ __forceinline__ bool newton_keep(double s, double p, double q, double f, double, double sn,
-                                            double)
-{
-    const double fn = sn * sn * sn + p * sn + q;
-    return fabs(fn) <= fabs(f);
-}
-__device__ __forceinline__ bool newton_keep(float s, float, float, float, float fp, float, float quot)
-{
-    return fabsf(quot * (3.0f * s - quot)) <= fp;
-}
-
 // Eq. update: theta_c - (h^2/6)(s_new - s).
 //   rule 1: s_new = largest root (the paper's update), Newton-polished;
 //   rule 0: one Newton step on the cubic from s, taken only right of the
-//           local minimum of f and kept only if |f| does not grow; else rule 1.
-template <typename T>
-__device__ __forceinline__ T point_update(T theta_c, T h2_6, T s, T p, T q, int rule)
+//           local minimum of f (s > sqrt(-p/3)) and kept only if |f| does not
+//           grow; else rule 1.
+// |f| after the step is taken in the cancellation-free form
+// f(s + d) = d^2 (3 s + d) for the Newton step d = -f / f', so the test is
+// |d| |3 s + d| <= f'; recomputing f(s + d) near convergence gives rounding
+// noise, which rejects good steps at random (and sent whole warps through the
+// root of the cubic: an FP64 sweep of 128^3 took 461 us, 209 us in this form;
+// at one FP64 operation per 64 FP32 ones its ~50 operations are ~197 us).
+
+// FP32, on the cubic s^3 + p s + q; the quotient is the fast reciprocal form
+// (2 ulp), whose result the defect correction refines
+__device__ __forceinline__ float cell_update(const Nb19<float> &n, float rhs, float ih2, float h2_6, int rule)
 {
-    T sn;
+    float s, p, q, sn;
+    cubic_coeffs(n, ih2, rhs, s, p, q);
     bool done = false;
-    if (rule == 0 && right_of_min(s, p)) {
-        const T f = s * s * s + p * s + q;
-        const T fp = T(3) * s * s + p;
-        const T quot = newton_quot(f, fp);
+    if (rule == 0 && s > 0.0f && 3.0f * s * s > -p) {
+        const float f = s * s * s + p * s + q;
+        const float fp = 3.0f * s * s + p;
+        const float quot = __fdividef(f, fp);
         sn = s - quot;
-        done = newton_keep(s, p, q, f, fp, sn, quot);
+        done = fabsf(quot * (3.0f * s - quot)) <= fp;
     }
     if (!done) sn = root_polished(p, q);
-    return theta_c - h2_6 * (sn - s);
+    return n.c - h2_6 * (sn - s);
+}
+
+// a / b for positive normal b, within 1 ulp (Newton's iteration for 1 / b, with
+// Markstein's remainder step for the quotient): the hardware's reciprocal
+// approximation, one Newton step on 1 / b (to ~40 bits) and one on the
+// quotient, whose remainder is exact in one fma.  Four FP64 operations and no
+// branch; FP64 operations are what the FP64 smoother waits for.
+__device__ __forceinline__ double div_pos(double a, double b)
+{
+    double r;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(b));
+    r = fma(r, fma(-b, r, 1.0), r);
+    const double q = a * r;
+    return fma(fma(-b, q, a), r, q);
+}
+
+// Rule 1 from A = I + H theta: the cubic of the traceless part, its largest
+// root; returns theta_c - (h^2/6)(root - tr A).  Out of line: rare under rule 0.
+static __device__ __noinline__ double root_update(double theta_c, double axx, double ayy, double azz, double hxy,
+                                                  double hyz, double hxz, double rhs, double h2_6)
+{
+    const double s = axx + ayy + azz, third = s * (1.0 / 3.0);
+    const double bxx = axx - third, byy = ayy - third, bzz = azz - third;
+    const double tr2 = bxx * bxx + byy * byy + bzz * bzz + 2.0 * (hxy * hxy + hyz * hyz + hxz * hxz);
+    const double detb = bxx * (byy * bzz - hyz * hyz) - hxy * (hxy * bzz - hyz * hxz)
+                      + hxz * (hxy * hyz - byy * hxz);
+    return theta_c - h2_6 * (root_polished(-4.5 * tr2, 27.0 * detb - 27.0 * rhs) - s);
+}
+
+// FP64, on A = I + H theta directly: with s = tr A and S = tr adj A the cubic
+// is f = 27 (det A - rhs) with f' = 9 S, so Newton's step is
+// tau = (det A - rhs) / S, theta_c += (h^2/2) tau (every diagonal entry of A
+// moves by -tau), kept when s > 0, S > 0 and |tau| |s - tau| <= S.  ~50 FP64
+// operations per cell; the tests run on the integer pipes (signs, and the
+// order of the bit patterns of two non-negative numbers).  resid (nullable):
+// rhs - det A.
+__device__ __forceinline__ double cell_update(const Nb19<double> &n, double rhs, double ih2, double h2_6, int rule,
+                                              double *resid = nullptr)
+{
+    const double axx = fma(fma(-2.0, n.c, n.xp + n.xm), ih2, 1.0);
+    const double ayy = fma(fma(-2.0, n.c, n.yp + n.ym), ih2, 1.0);
+    const double azz = fma(fma(-2.0, n.c, n.zp + n.zm), ih2, 1.0);
+    double hxy, hyz, hxz;
+    mixed(n, ih2 * 0.25, hxy, hyz, hxz);
+    const double cxx = fma(-hyz, hyz, ayy * azz);
+    const double cyy = fma(-hxz, hxz, axx * azz);
+    const double czz = fma(-hxy, hxy, axx * ayy);
+    const double cxy = fma(hxz, hyz, -(hxy * azz));
+    const double cxz = fma(hxy, hyz, -(hxz * ayy));
+    const double F = fma(axx, cxx, fma(hxy, cxy, fma(hxz, cxz, -rhs)));
+    if (resid) *resid = -F;
+    const double S = cxx + cyy + czz, s = axx + ayy + azz;
+    const double tau = div_pos(F, S), u = tau * (s - tau);
+    const long long ub = __double_as_longlong(u) & 0x7fffffffffffffffll;
+    if (rule == 0 && __double_as_longlong(s) > 0 && ub <= __double_as_longlong(S))   // (u a NaN: false)
+        return fma(tau, 3.0 * h2_6, n.c);
+    return root_update(n.c, axx, ayy, azz, hxy, hyz, hxz, rhs, h2_6);
 }
 
 }  // namespace recon

@@ -61,12 +61,10 @@ k_rb_pass(const T *__restrict__ src, T *__restrict__ dst, const T *__restrict__ 
     {
         const int par = (colour + i + j) & 1;   // (i + j + k) % 2 == colour
         const unsigned base = offs(N, i, j, 0);
-        for (int m = threadIdx.x; m < half; m += kRowX) {
+        for (int m = threadIdx.x; m < half; m += blockDim.x) {
             const int ka = 2 * m + par, kb = 2 * m + 1 - par;
             const Nb19<T> nb = load19<T>(src, N, i, j, ka);
-            T s, p, q;
-            cubic_coeffs(nb, ih2, g[base + ka] + c, s, p, q);
-            dst[base + ka] = point_update(nb.c, h2_6, s, p, q, rule);
+            dst[base + ka] = cell_update(nb, g[base + ka] + c, ih2, h2_6, rule);
             dst[base + kb] = src[base + kb];
         }
     }
@@ -124,10 +122,10 @@ static_assert(kTK / 2 == 32 && kRH == 33 && kWarps == 8 && kTJ == 2 * kWarps,
               "warp w owns tile rows w and w + 8 and red index = lane");
 static_assert(kRJ - 2 * kWarps == 2, "RED rows 16 and 17 go to warps 0 and 1");
 
-template <typename T, bool LIN>
+template <bool LIN>
 constexpr size_t fused_smem_bytes()
 {
-    return sizeof(T) * (size_t)(red_base<LIN>() + kRSlots * kRPlane);
+    return sizeof(float) * (size_t)(red_base<LIN>() + kRSlots * kRPlane);
 }
 
 __device__ __forceinline__ int wrap1(int x, int N) { return x < 0 ? x + N : (x >= N ? x - N : x); }
@@ -147,11 +145,6 @@ __device__ __forceinline__ void cp_async_elem(float *sdst, const float *gsrc)
     const unsigned sa = (unsigned)__cvta_generic_to_shared(sdst);
     asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(sa), "l"(gsrc));
 }
-__device__ __forceinline__ void cp_async_elem(double *sdst, const double *gsrc)
-{
-    const unsigned sa = (unsigned)__cvta_generic_to_shared(sdst);
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(sa), "l"(gsrc));
-}
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::); }
 template <int K>
 __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;\n" ::"n"(K)); }
@@ -160,10 +153,9 @@ __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_gr
 // element offsets pm, pc, pp of the shared buffer sm.  S: the cell's offset
 // within a plane (its own parity half); O: the offset of its k-1 neighbour
 // (other half), k+1 being O + 1.
-template <typename T>
-__device__ __forceinline__ Nb19<T> gather19(const T *sm, int pm, int pc, int pp, int S, int O)
+__device__ __forceinline__ Nb19<float> gather19(const float *sm, int pm, int pc, int pp, int S, int O)
 {
-    Nb19<T> v;
+    Nb19<float> v;
     v.c = sm[pc + S];
     v.xp = sm[pp + S];
     v.xm = sm[pm + S];
@@ -219,44 +211,29 @@ __device__ __forceinline__ void gather19_il(const float *sm, int pm, int pc, int
     ld(pp + O, e.xpzm, t.xpzm);
 }
 
-// The nonlinear cell update (eq. update).
-template <typename T>
-__device__ __forceinline__ T fas_update(const Nb19<T> &nb, T rhs, T ih2, T h2_6, int rule)
-{
-    T s, p, q;
-    cubic_coeffs(nb, ih2, rhs, s, p, q);
-    return point_update(nb.c, h2_6, s, p, q, rule);
-}
-
 // Gauss-Seidel on J e = f at a cell: J = sum_ab adj(I + H theta)_ab D_ab,
 // J_cc = -2 (adj_xx + adj_yy + adj_zz) / h^2.
-template <typename T>
-__device__ __forceinline__ T lin_update(const Nb19<T> &nt, const Nb19<T> &ne, T rhs, T ih2)
+__device__ __forceinline__ float lin_update(const Nb19<float> &nt, const Nb19<float> &ne, float rhs, float ih2)
 {
-    const Cof<T> a = cofactors(nt, ih2);
-    const T Je = jac_apply(a, ne, ih2);
-    const T diag = T(-2) * (a.xx + a.yy + a.zz) * ih2;
+    const Cof<float> a = cofactors(nt, ih2);
+    const float Je = jac_apply(a, ne, ih2);
+    const float diag = -2.0f * (a.xx + a.yy + a.zz) * ih2;
     return ne.c + (rhs - Je) / diag;
 }
 
-template <typename T> struct Pair;
-template <> struct Pair<float> { using type = float2; };
-template <> struct Pair<double> { using type = double2; };
-
-template <typename T, bool LIN>
-// CTAs per SM: FP64 2 (registers), linear 3 (shared memory), FP32 FAS 4
-// (64 registers for the paired updates without spills)
-__global__ void __launch_bounds__(kFT, sizeof(T) == 8 ? 2 : (LIN ? 3 : 4))
-k_sweep_fused(const T *__restrict__ src, T *__restrict__ dst, const T *__restrict__ g,
-              const T *__restrict__ th, const double *__restrict__ cptr, double cval, int N,
-              int CI, T ih2, T h2_6, int rule)
+template <bool LIN>
+// CTAs per SM: linear 3 (shared memory), FAS 4 (64 registers for the paired
+// updates without spills)
+__global__ void __launch_bounds__(kFT, LIN ? 3 : 4)
+k_sweep_fused(const float *__restrict__ src, float *__restrict__ dst, const float *__restrict__ g,
+              const float *__restrict__ th, const double *__restrict__ cptr, double cval, int N,
+              int CI, float ih2, float h2_6, int rule)
 {
-    // FP32: a thread's two rows 8 apart are relaxed together with paired
-    // FP32 instructions (cellmath2.cuh); FP64 relaxes them one by one
-    constexpr bool kPaired = std::is_same<T, float>::value;
+    // a thread's two rows 8 apart are relaxed together with paired FP32
+    // instructions (cellmath2.cuh)
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    T *sm = reinterpret_cast<T *>(smem_raw);
-    const T c = LIN ? T(0) : (T)(cptr ? *cptr : cval);
+    float *sm = reinterpret_cast<float *>(smem_raw);
+    const float c = LIN ? float(0) : (float)(cptr ? *cptr : cval);
     const int k0 = blockIdx.x * kTK, j0 = blockIdx.y * kTJ, i0 = blockIdx.z * CI;
     const int i1 = min(i0 + CI, N);
     const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
@@ -280,7 +257,7 @@ k_sweep_fused(const T *__restrict__ src, T *__restrict__ dst, const T *__restric
 #pragma unroll
             for (int t = 0; t < kLoadsPerThread; ++t)
                 if (soff[t] >= 0) {
-                    T *d = sm + 2 * (slot + soff[t]);
+                    float *d = sm + 2 * (slot + soff[t]);
                     cp_async_elem(d, src + pb + goff[t]);
                     cp_async_elem(d + 1, th + pb + goff[t]);
                 }
@@ -314,36 +291,35 @@ k_sweep_fused(const T *__restrict__ src, T *__restrict__ dst, const T *__restric
         const int S0 = (w + 1) * kOR + (pr ^ 1) * kOH + lane + pr;
         const int O0 = (w + 1) * kOR + pr * kOH + lane;
         const unsigned gc = pb + (pr ? gcol1 : gcol0);
-        if constexpr (kPaired) {
+        {
             // RED rows w and w + 8 as one pair of paired-FP32 updates
             constexpr int D = 8 * kOR;
             const float2 rhs = make_float2(g[gc + grow[0]], g[gc + grow[1]]);
             float2 v;
             if constexpr (LIN) {
-                Nb19<T> ea, ta, eb, tb;
+                Nb19<float> ea, ta, eb, tb;
                 gather19_il(sm, om, oc, op, S0, O0, ea, ta);
                 gather19_il(sm, om, oc, op, S0 + D, O0 + D, eb, tb);
-                v = lin_update2(pack19(ta, tb), pack19(ea, eb), rhs, ih2, T(6) * h2_6);
+                v = lin_update2(pack19(ta, tb), pack19(ea, eb), rhs, ih2, float(6) * h2_6);
             } else {
-                const Nb19<float2> nb = pack19(gather19<T>(sm, om, oc, op, S0, O0),
-                                               gather19<T>(sm, om, oc, op, S0 + D, O0 + D));
+                const Nb19<float2> nb = pack19(gather19(sm, om, oc, op, S0, O0),
+                                               gather19(sm, om, oc, op, S0 + D, O0 + D));
                 v = fas_update2(nb, add2(rhs, f2(c)), ih2, h2_6, rule);
             }
             sm[rs + w * kRH + lane] = v.x;
             sm[rs + (w + 8) * kRH + lane] = v.y;
         }
-#pragma unroll
-        for (int i = kPaired ? 2 : 0; i < 3; ++i) {
-            if (i == 2 && w >= kRJ - 2 * kWarps) break;
+        if (w < kRJ - 2 * kWarps) {   // RED rows 16 and 17
+            constexpr int i = 2;
             const int S = S0 + 8 * i * kOR, O = O0 + 8 * i * kOR;
-            const T rhs = g[gc + grow[i]];
-            T v;
+            const float rhs = g[gc + grow[i]];
+            float v;
             if constexpr (LIN) {
-                Nb19<T> e, t;
+                Nb19<float> e, t;
                 gather19_il(sm, om, oc, op, S, O, e, t);
-                v = lin_update<T>(t, e, rhs, ih2);
+                v = lin_update(t, e, rhs, ih2);
             } else {
-                v = fas_update<T>(gather19<T>(sm, om, oc, op, S, O), rhs + c, ih2, h2_6, rule);
+                v = cell_update(gather19(sm, om, oc, op, S, O), rhs + c, ih2, h2_6, rule);
             }
             sm[rs + (w + 8 * i) * kRH + lane] = v;
         }
@@ -351,14 +327,14 @@ k_sweep_fused(const T *__restrict__ src, T *__restrict__ dst, const T *__restric
             const int r = lane, prc = (p + j0 + r) & 1, h = kRH - 1;
             const int S = (r + 1) * kOR + (prc ^ 1) * kOH + h + prc;
             const int O = (r + 1) * kOR + prc * kOH + h;
-            const T rhs = g[pb + crow + (prc ? ccol1 : ccol0)];
-            T v;
+            const float rhs = g[pb + crow + (prc ? ccol1 : ccol0)];
+            float v;
             if constexpr (LIN) {
-                Nb19<T> e, t;
+                Nb19<float> e, t;
                 gather19_il(sm, om, oc, op, S, O, e, t);
-                v = lin_update<T>(t, e, rhs, ih2);
+                v = lin_update(t, e, rhs, ih2);
             } else {
-                v = fas_update<T>(gather19<T>(sm, om, oc, op, S, O), rhs + c, ih2, h2_6, rule);
+                v = cell_update(gather19(sm, om, oc, op, S, O), rhs + c, ih2, h2_6, rule);
             }
             sm[rs + r * kRH + h] = v;
         }
@@ -375,77 +351,44 @@ k_sweep_fused(const T *__restrict__ src, T *__restrict__ dst, const T *__restric
         const int Q0 = (w + 1) * kRH + lane;
         const unsigned sb = (unsigned)s * NN;
         const int gk0 = k0 + 2 * lane;
-        if constexpr (kPaired) {
-            // tile rows w and w + 8 as one pair of paired-FP32 updates; a
-            // row or column outside the grid (ragged tile) is computed from
-            // the wrapped halo values but neither read from g nor stored
-            constexpr int D = 8 * kOR, DR = 8 * kRH;
-            const int gj = j0 + w;
-            const bool in0 = gk0 < N && gj < N, in1 = gk0 < N && gj + 8 < N;
-            Nb19<T> a, b, ta, tb;   // ta, tb: theta (linear smoother)
-            if constexpr (LIN) {
-                gather19_il(sm, om, oc, op, S0, O0, a, ta);
-                gather19_il(sm, om, oc, op, S0 + D, O0 + D, b, tb);
-            } else {
-                a = gather19<T>(sm, om, oc, op, S0, O0);
-                b = gather19<T>(sm, om, oc, op, S0 + D, O0 + D);
-            }
-            a.xp = sm[rp + Q0 + pb];
-            a.xm = sm[rm + Q0 + pb];
-            a.yp = sm[rc + Q0 + kRH + pb];
-            a.ym = sm[rc + Q0 - kRH + pb];
-            a.zp = sm[rc + Q0 + 1];
-            a.zm = sm[rc + Q0];
-            b.xp = sm[rp + Q0 + DR + pb];
-            b.xm = sm[rm + Q0 + DR + pb];
-            b.yp = sm[rc + Q0 + DR + kRH + pb];
-            b.ym = sm[rc + Q0 + DR - kRH + pb];
-            b.zp = sm[rc + Q0 + DR + 1];
-            b.zm = sm[rc + Q0 + DR];
-            const unsigned gb0 = sb + (unsigned)gj * (unsigned)N + (unsigned)gk0;
-            const unsigned gb1 = gb0 + 8u * (unsigned)N;
-            const float2 rhs = make_float2(in0 ? g[gb0 + pb] : T(1), in1 ? g[gb1 + pb] : T(1));
-            float2 vb;
-            if constexpr (LIN) {
-                vb = lin_update2(pack19(ta, tb), pack19(a, b), rhs, ih2, T(6) * h2_6);
-            } else {
-                vb = fas_update2(pack19(a, b), add2(rhs, f2(c)), ih2, h2_6, rule);
-            }
-            const T vr0 = sm[rc + Q0 + 1 - pb], vr1 = sm[rc + Q0 + DR + 1 - pb];
-            if (in0) *reinterpret_cast<float2 *>(dst + gb0) = pb ? make_float2(vr0, vb.x) : make_float2(vb.x, vr0);
-            if (in1) *reinterpret_cast<float2 *>(dst + gb1) = pb ? make_float2(vr1, vb.y) : make_float2(vb.y, vr1);
+        // tile rows w and w + 8 as one pair of paired-FP32 updates; a
+        // row or column outside the grid (ragged tile) is computed from
+        // the wrapped halo values but neither read from g nor stored
+        constexpr int D = 8 * kOR, DR = 8 * kRH;
+        const int gj = j0 + w;
+        const bool in0 = gk0 < N && gj < N, in1 = gk0 < N && gj + 8 < N;
+        Nb19<float> a, b, ta, tb;   // ta, tb: theta (linear smoother)
+        if constexpr (LIN) {
+            gather19_il(sm, om, oc, op, S0, O0, a, ta);
+            gather19_il(sm, om, oc, op, S0 + D, O0 + D, b, tb);
         } else {
-#pragma unroll
-            for (int i = 0; i < 2; ++i) {
-                const int gj = j0 + w + 8 * i;
-                if (gj >= N || gk0 >= N) continue;
-                const int S = S0 + 8 * i * kOR, O = O0 + 8 * i * kOR, Q = Q0 + 8 * i * kRH;
-                Nb19<T> nb, nt;   // nt: theta (linear smoother)
-                if constexpr (LIN) {
-                    gather19_il(sm, om, oc, op, S, O, nb, nt);
-                } else {
-                    nb = gather19<T>(sm, om, oc, op, S, O);
-                }
-                nb.xp = sm[rp + Q + pb];
-                nb.xm = sm[rm + Q + pb];
-                nb.yp = sm[rc + Q + kRH + pb];
-                nb.ym = sm[rc + Q - kRH + pb];
-                nb.zp = sm[rc + Q + 1];
-                nb.zm = sm[rc + Q];
-                const unsigned gb = sb + (unsigned)gj * (unsigned)N + (unsigned)gk0;
-                T vb;
-                if constexpr (LIN) {
-                    vb = lin_update<T>(nt, nb, g[gb + pb], ih2);
-                } else {
-                    vb = fas_update<T>(nb, g[gb + pb] + c, ih2, h2_6, rule);
-                }
-                const T vr = sm[rc + Q + 1 - pb];
-                typename Pair<T>::type v;
-                v.x = pb ? vr : vb;
-                v.y = pb ? vb : vr;
-                *reinterpret_cast<typename Pair<T>::type *>(dst + gb) = v;
-            }
+            a = gather19(sm, om, oc, op, S0, O0);
+            b = gather19(sm, om, oc, op, S0 + D, O0 + D);
         }
+        a.xp = sm[rp + Q0 + pb];
+        a.xm = sm[rm + Q0 + pb];
+        a.yp = sm[rc + Q0 + kRH + pb];
+        a.ym = sm[rc + Q0 - kRH + pb];
+        a.zp = sm[rc + Q0 + 1];
+        a.zm = sm[rc + Q0];
+        b.xp = sm[rp + Q0 + DR + pb];
+        b.xm = sm[rm + Q0 + DR + pb];
+        b.yp = sm[rc + Q0 + DR + kRH + pb];
+        b.ym = sm[rc + Q0 + DR - kRH + pb];
+        b.zp = sm[rc + Q0 + DR + 1];
+        b.zm = sm[rc + Q0 + DR];
+        const unsigned gb0 = sb + (unsigned)gj * (unsigned)N + (unsigned)gk0;
+        const unsigned gb1 = gb0 + 8u * (unsigned)N;
+        const float2 rhs = make_float2(in0 ? g[gb0 + pb] : float(1), in1 ? g[gb1 + pb] : float(1));
+        float2 vb;
+        if constexpr (LIN) {
+            vb = lin_update2(pack19(ta, tb), pack19(a, b), rhs, ih2, float(6) * h2_6);
+        } else {
+            vb = fas_update2(pack19(a, b), add2(rhs, f2(c)), ih2, h2_6, rule);
+        }
+        const float vr0 = sm[rc + Q0 + 1 - pb], vr1 = sm[rc + Q0 + DR + 1 - pb];
+        if (in0) *reinterpret_cast<float2 *>(dst + gb0) = pb ? make_float2(vr0, vb.x) : make_float2(vb.x, vr0);
+        if (in1) *reinterpret_cast<float2 *>(dst + gb1) = pb ? make_float2(vr1, vb.y) : make_float2(vb.y, vr1);
     };
 
     // prologue: OLD planes i0-2 .. i0+2 into slots 0..4, then RED planes
@@ -484,11 +427,11 @@ k_sweep_fused(const T *__restrict__ src, T *__restrict__ dst, const T *__restric
     cp_async_wait<0>();
 }
 
-template <typename T, bool LIN>
+template <bool LIN>
 static cudaError_t fused_attr()
 {
-    return cudaFuncSetAttribute(k_sweep_fused<T, LIN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)fused_smem_bytes<T, LIN>());
+    return cudaFuncSetAttribute(k_sweep_fused<LIN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                (int)fused_smem_bytes<LIN>());
 }
 
 static bool g_kernels_ready = false;
@@ -500,9 +443,8 @@ void set_fused_chunk(int c) { g_fused_chunk = c; }
 
 cudaError_t prepare_kernels()
 {
-    cudaError_t e = fused_attr<float, false>();
-    if (e == cudaSuccess) e = fused_attr<double, false>();
-    if (e == cudaSuccess) e = fused_attr<float, true>();
+    cudaError_t e = fused_attr<false>();
+    if (e == cudaSuccess) e = fused_attr<true>();
     if (e == cudaSuccess) e = prepare_reg_sweeps();
     if (e == cudaSuccess) e = coarse_attrs();
     if (e == cudaSuccess) e = prepare_tails();
@@ -513,21 +455,20 @@ cudaError_t prepare_kernels()
 // The fused sweeps store (even k, odd k) pairs as one vector: the arrays they
 // write must be aligned to two elements (true of every allocation; a caller's
 // offset view may not be, and then the two-pass kernels run instead).
-template <typename T>
-static inline bool pair_aligned(const T *p)
+static inline bool pair_aligned(const float *p)
 {
-    return ((uintptr_t)p % (2 * sizeof(T))) == 0;
+    return ((uintptr_t)p % (2 * sizeof(float))) == 0;
 }
 
 // th: the theta of the linear variant (nullptr for the nonlinear one)
-template <typename T, bool LIN>
-static cudaError_t fused_sweep_launch(int N, const T *src, T *dst, const T *g, const T *th,
-                                      const double *cptr, double cval, T ih2, T h2_6, int rule,
+template <bool LIN>
+static cudaError_t fused_sweep_launch(int N, const float *src, float *dst, const float *g, const float *th,
+                                      const double *cptr, double cval, float ih2, float h2_6, int rule,
                                       cudaStream_t s)
 {
     // set once per process (recon_create does it before any graph capture;
     // step entry points may run without a handle)
-    const size_t smem = fused_smem_bytes<T, LIN>();
+    const size_t smem = fused_smem_bytes<LIN>();
     if (!g_kernels_ready) {
         const cudaError_t e = prepare_kernels();
         if (e != cudaSuccess) return e;
@@ -535,7 +476,7 @@ static cudaError_t fused_sweep_launch(int N, const T *src, T *dst, const T *g, c
     const int CI = g_fused_chunk > 0 ? g_fused_chunk : (N >= 512 ? 64 : (N >= 256 ? 32 : 16));
     const dim3 grid((N + kTK - 1) / kTK, (N + kTJ - 1) / kTJ, (N + CI - 1) / CI);
     note_launch();
-    k_sweep_fused<T, LIN><<<grid, kFT, smem, s>>>(src, dst, g, th, cptr, cval, N, CI, ih2, h2_6, rule);
+    k_sweep_fused<LIN><<<grid, kFT, smem, s>>>(src, dst, g, th, cptr, cval, N, CI, ih2, h2_6, rule);
     return cudaGetLastError();
 }
 
@@ -563,22 +504,29 @@ cudaError_t sweep(int N, double h, int rule, T *t, const T *g, const double *cpt
         note_launch();
         k_gauge_by<T><<<stride_blocks((size_t)N * N * N), kThreads, 0, s>>>(t, (size_t)N * N * N, gshift);
     }
-    if (N >= kFusedMinN && pair_aligned(t) && pair_aligned(work)) {
-        T *a = t, *b = work;
-        for (int it = 0; it < sweeps; ++it) {
-            const cudaError_t e = fused_sweep_launch<T, false>(N, a, b, g, (const T *)nullptr, cptr, cval, ih2, h2_6, rule, s);
-            if (e != cudaSuccess) return e;
-            T *tmp = a;
-            a = b;
-            b = tmp;
+    // FP64 stays on the two-pass kernels at every size: the FP64 pipe bounds
+    // both forms, and the fused one recomputes the red cells of its tiles'
+    // rings (measured per sweep: 128^3 209 us against 271 fused, 256^3 1.55
+    // against 1.99 ms, 512^3 12.3 against 13.6 ms)
+    if constexpr (std::is_same<T, float>::value) {
+        if (N >= kFusedMinN && pair_aligned(t) && pair_aligned(work)) {
+            float *a = t, *b = work;
+            for (int it = 0; it < sweeps; ++it) {
+                const cudaError_t e = fused_sweep_launch<false>(N, a, b, g, nullptr, cptr, cval, ih2, h2_6, rule, s);
+                if (e != cudaSuccess) return e;
+                float *tmp = a;
+                a = b;
+                b = tmp;
+            }
+            if (a != t) return cudaMemcpyAsync(t, a, sizeof(float) * (size_t)N * N * N, cudaMemcpyDeviceToDevice, s);
+            return cudaSuccess;
         }
-        if (a != t) return cudaMemcpyAsync(t, a, sizeof(T) * (size_t)N * N * N, cudaMemcpyDeviceToDevice, s);
-        return cudaSuccess;
     }
+    const dim3 fit = fit_block(N / 2);
     for (int it = 0; it < sweeps; ++it) {
         note_launch(2);
-        k_rb_pass<T><<<row_grid(N), row_block(), 0, s>>>(t, work, g, cptr, cval, N, ih2, h2_6, 0, rule);
-        k_rb_pass<T><<<row_grid(N), row_block(), 0, s>>>(work, t, g, cptr, cval, N, ih2, h2_6, 1, rule);
+        k_rb_pass<T><<<fit_grid(N, fit), fit, 0, s>>>(t, work, g, cptr, cval, N, ih2, h2_6, 0, rule);
+        k_rb_pass<T><<<fit_grid(N, fit), fit, 0, s>>>(work, t, g, cptr, cval, N, ih2, h2_6, 1, rule);
     }
     return cudaGetLastError();
 }
@@ -982,13 +930,16 @@ k_prolong_add(const T *__restrict__ cnew, const T *__restrict__ cold, int Nc,
     using V2 = typename Vec2<T>::type;
     const double sc = pscale ? *pscale : scale;
     if (sc == 0.0) return;
-    const T s = (T)sc, w0 = T(0.75), w1 = T(0.25);
+    // per axis the weights 3/4, 1/4 as 3 a + b, all three quarters in the scale
+    // (exact): one operation per interpolated value, which is what the FP64
+    // form waits for (FP64 128^3: 69 -> 41 us)
+    const T s = (T)(sc * (1.0 / 64.0));
     const int Nf = 2 * Nc;
     FOR_ROWS(Nc, I, J)
     {
         const int Ip[3] = {I == 0 ? Nc - 1 : I - 1, I, I + 1 == Nc ? 0 : I + 1};
         const int Jp[3] = {J == 0 ? Nc - 1 : J - 1, J, J + 1 == Nc ? 0 : J + 1};
-        for (int K = threadIdx.x; K < Nc; K += kRowX) {
+        for (int K = threadIdx.x; K < Nc; K += blockDim.x) {
             const int Kp[3] = {K == 0 ? Nc - 1 : K - 1, K, K + 1 == Nc ? 0 : K + 1};
             // the four fine pairs first: their DRAM reads overlap the coarse loads
             unsigned fo[2][2];
@@ -1021,15 +972,15 @@ k_prolong_add(const T *__restrict__ cnew, const T *__restrict__ cold, int Nc,
 #pragma unroll
                 for (int b = 0; b < 3; ++b)
 #pragma unroll
-                    for (int c = 0; c < 3; ++c) u[b][c] = w0 * d[1][b][c] + w1 * d[ei ? 2 : 0][b][c];
+                    for (int c = 0; c < 3; ++c) u[b][c] = fma(T(3), d[1][b][c], d[ei ? 2 : 0][b][c]);
 #pragma unroll
                 for (int ej = 0; ej < 2; ++ej) {
                     T v[3];
 #pragma unroll
-                    for (int c = 0; c < 3; ++c) v[c] = w0 * u[1][c] + w1 * u[ej ? 2 : 0][c];
+                    for (int c = 0; c < 3; ++c) v[c] = fma(T(3), u[1][c], u[ej ? 2 : 0][c]);
                     V2 x = fv[ei][ej];
-                    x.x += s * (w0 * v[1] + w1 * v[0]);
-                    x.y += s * (w0 * v[1] + w1 * v[2]);
+                    x.x = fma(s, fma(T(3), v[1], v[0]), x.x);
+                    x.y = fma(s, fma(T(3), v[1], v[2]), x.y);
                     if (pairs) {
                         *reinterpret_cast<V2 *>(fine + fo[ei][ej]) = x;
                     } else {
@@ -1048,7 +999,8 @@ cudaError_t prolong_add(int Nc, const T *cnew, const T *cold, const double *psca
 {
     note_launch();
     const int pairs = ((uintptr_t)fine % (2 * sizeof(T))) == 0;
-    k_prolong_add<T><<<row_grid(Nc), row_block(), 0, s>>>(cnew, cold, Nc, pscale, scale, fine, pairs);
+    const dim3 fit = fit_block(Nc);
+    k_prolong_add<T><<<fit_grid(Nc, fit), fit, 0, s>>>(cnew, cold, Nc, pscale, scale, fine, pairs);
     return cudaGetLastError();
 }
 template cudaError_t prolong_add<double>(int, const double *, const double *, const double *, double, double *, cudaStream_t);
@@ -1124,9 +1076,7 @@ k_coarse_solve(T *t, T *work, const T *g, const double *cptr, double cval, int N
                 const int par = (colour + i + j) & 1;
                 const int ka = 2 * m + par, kb = 2 * m + 1 - par;
                 const Nb19<T> nb = load19<T>(src, N, i, j, ka);
-                T s, p, q;
-                cubic_coeffs(nb, ih2, gs[offs(N, i, j, ka)] + c, s, p, q);
-                const T vnew = point_update(nb.c, h2_6, s, p, q, rule);
+                const T vnew = cell_update(nb, gs[offs(N, i, j, ka)] + c, ih2, h2_6, rule);
                 const T vcopy = src[offs(N, i, j, kb)];
                 dst[offs(N, i, j, ka)] = vnew;
                 dst[offs(N, i, j, kb)] = vcopy;
@@ -1426,7 +1376,7 @@ k_lin_pass(const float *__restrict__ src, float *__restrict__ dst, const float *
     {
         const int par = (colour + i + j) & 1;
         const unsigned base = offs(N, i, j, 0);
-        for (int m = threadIdx.x; m < half; m += kRowX) {
+        for (int m = threadIdx.x; m < half; m += blockDim.x) {
             const int ka = 2 * m + par, kb = 2 * m + 1 - par;
             const Cof<float> a = cof_at(cof, n, cof_slot(N, i, j, ka));
             const Nb19<float> ev = load19<float>(src, N, i, j, ka);
@@ -1468,7 +1418,7 @@ static cudaError_t lin_sweep(int N, double h, float *e, const float *f, const fl
     if (lin_fused(N, e, work)) {
         float *a = e, *b = work;
         for (int it = 0; it < sweeps; ++it) {
-            const cudaError_t err = fused_sweep_launch<float, true>(N, a, b, f, th, nullptr, 0.0, ih2,
+            const cudaError_t err = fused_sweep_launch<true>(N, a, b, f, th, nullptr, 0.0, ih2,
                                                                    (float)(h * h / 6.0), 0, s);
             if (err != cudaSuccess) return err;
             float *tmp = a;
@@ -1478,10 +1428,11 @@ static cudaError_t lin_sweep(int N, double h, float *e, const float *f, const fl
         if (a != e) return cudaMemcpyAsync(e, a, sizeof(float) * (size_t)N * N * N, cudaMemcpyDeviceToDevice, s);
         return cudaSuccess;
     }
+    const dim3 fit = fit_block(N / 2);
     for (int it = 0; it < sweeps; ++it) {
         note_launch(2);
-        k_lin_pass<<<row_grid(N), row_block(), 0, s>>>(e, work, f, cof, N, ih2, 0);
-        k_lin_pass<<<row_grid(N), row_block(), 0, s>>>(work, e, f, cof, N, ih2, 1);
+        k_lin_pass<<<fit_grid(N, fit), fit, 0, s>>>(e, work, f, cof, N, ih2, 0);
+        k_lin_pass<<<fit_grid(N, fit), fit, 0, s>>>(work, e, f, cof, N, ih2, 1);
     }
     return cudaGetLastError();
 }

@@ -85,9 +85,7 @@ k_slab_pass(const double *__restrict__ src, double *__restrict__ dst, const doub
             continue;
         }
         const Nb19<double> n = load19s(src, S, i, j, k);
-        double s, p, q;
-        cubic_coeffs(n, ih2, g[id] + c, s, p, q);
-        dst[id] = point_update(n.c, h2_6, s, p, q, rule);
+        dst[id] = cell_update(n, g[id] + c, ih2, h2_6, rule);
     }
 }
 

@@ -115,18 +115,12 @@ struct Math<double> {
     static __device__ __forceinline__ bool le(V a, V b) { return a <= b; }
     static __device__ __forceinline__ double round(V a) { return a; }
     static __device__ __forceinline__ double get(V a) { return a; }
-    static __device__ __forceinline__ double one(const Nb19<double> &n, double r, double ih2, double h2_6, int rule)
-    {
-        double s, p, q;
-        cubic_coeffs(n, ih2, r, s, p, q);
-        return point_update(n.c, h2_6, s, p, q, rule);
-    }
     static __device__ __forceinline__ void update(const Nb19<double> &a, const Nb19<double> &b, double ra, double rb,
                                                   double ih2, double h2_6, int rule, bool two, double &va, double &vb,
-                                                  double &, double &)
+                                                  double &fa, double &fb)
     {
-        va = one(a, ra, ih2, h2_6, rule);
-        if (two) vb = one(b, rb, ih2, h2_6, rule);
+        va = cell_update(a, ra, ih2, h2_6, rule, &fa);
+        if (two) vb = cell_update(b, rb, ih2, h2_6, rule, &fb);
     }
     static __device__ __forceinline__ void det(const Nb19<double> &a, const Nb19<double> &b, double ih2, bool two,
                                                double &da, double &db)
@@ -756,12 +750,7 @@ __global__ void __launch_bounds__(NT, 1) k_fas_tail(const __grid_constant__ Tail
                 const T ga = g_at(G, w, kr) + c, gb = g_at(G, w, kb) + c;
                 T va, vb;
                 M::update(a, b, ga, gb, A.ih2[G.l], A.h2_6[G.l], A.rule, false, va, vb, rr, rb);
-                if constexpr (sizeof(T) == 8) {
-                    T da, db;
-                    M::det(a, b, A.ih2[G.l], true, da, db);
-                    rr = ga - da;
-                    rb = gb - db;
-                }
+                if constexpr (sizeof(T) == 8) rb = gb - det_IH(b, A.ih2[G.l]);
                 return va;
             },
             [&](int src, const Row &w, int kb) {
