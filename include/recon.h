@@ -96,8 +96,9 @@ typedef struct {
     int adjoint_store_cofactors; /* recon_adjoint: 0 = the finest grid's six
                                    cofactor fields of I + H phi are formed
                                    again from phi in every application of J^T
-                                   (grids of side a multiple of 32; saves 48 N^3
-                                   bytes); 1 = kept in memory (faster)          */
+                                   (grids of side a multiple of 32; saves 72 N^3
+                                   bytes: FP64 and FP32 copies); 1 = kept in
+                                   memory                                       */
     int report_paper_eps;       /* recon_solve: 1 = fill recon_stats.paper_eps
                                    (one FP64 pass with the cubic's largest root
                                    per cell: ~0.3 s at 512^3); 0 = NaN         */
@@ -282,6 +283,9 @@ recon_status recon_gaussianise(recon_handle *h, const double *field, double *out
  * on (*)): given gbar_phi = dLoss/dphi (device N^3), writes
  * gbar_b = dLoss/db (device N^3, zero-sum), i.e. lam with
  *   J^T lam + mu 1 = gbar_phi,  sum(lam) = 0,  J = d det(I + H phi)/d phi.
+ * lam and the residual of this equation are FP64, to a relative residual of
+ * 1e-12; on grids above 32^3 the corrections between two residuals are FP32
+ * multigrid cycles (FP64 ones where those do not get there).
  * Errors: RECON_E_INVALID (no previous solve), RECON_E_NOCONV,
  * RECON_E_CUDA, RECON_E_UNIMPLEMENTED (not available in this build). */
 recon_status recon_adjoint(recon_handle *h, const double *gbar_phi, double *gbar_b);

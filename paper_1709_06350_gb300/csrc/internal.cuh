@@ -29,6 +29,10 @@ struct AdjWork {
     double null_rel = 0.0;
     double *th[kMaxLevels] = {}, *cof[kMaxLevels] = {}, *lam[kMaxLevels] = {}, *f[kMaxLevels] = {};
     double *nvec = nullptr;
+    // FP32 corrections: levels 1.. (cof32[0] if stored0)
+    float *cof32[kMaxLevels] = {}, *lam32[kMaxLevels] = {}, *f32[kMaxLevels] = {};
+    bool cof32_ready = false, cof64_ready = false;   // cofactors match the last solve
+    bool ready64 = false;      // the FP64 coarse levels are allocated
 };
 
 struct recon_handle {
@@ -139,9 +143,12 @@ bool tail_ok(int N);
 // level's scale factor is left in its scalar slots
 template <typename T>
 cudaError_t fas_tail(recon_handle *H, int l, T *t, const T *g, const double *cptr, bool raw);
-// the linear V-cycle from level l down on e32, f32 (levels with stored
-// cofactors).  raw: f's mean is removed first; zero: e starts from 0
-cudaError_t lin_tail(recon_handle *H, int l, bool raw, bool zero);
+// the linear V-cycle J e = f from level l down; cof: the colour-split
+// cofactors of every level of the hierarchy.  raw: f's mean is removed first;
+// zero: e starts from 0
+cudaError_t lin_tail(recon_handle *H, int l, float *e, const float *f, const float *const *cof, bool raw, bool zero);
+// six colour-split cofactor arrays of I + H theta (recon_mg.cu)
+cudaError_t cof6_split(int N, double h, const float *th, float *cof, cudaStream_t s);
 
 // ---- the solvers (recon_mg.cu)
 recon_status solve_f64(recon_handle *H, const double *b, double *phi, double tol,

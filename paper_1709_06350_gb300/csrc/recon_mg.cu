@@ -1352,6 +1352,13 @@ k_cof6f(const float *__restrict__ th, int N, float ih2, float *__restrict__ cof)
     }
 }
 
+cudaError_t cof6_split(int N, double h, const float *th, float *cof, cudaStream_t s)
+{
+    note_launch();
+    k_cof6f<<<row_grid(N), row_block(), 0, s>>>(th, N, (float)(1.0 / (h * h)), cof);
+    return cudaGetLastError();
+}
+
 __device__ __forceinline__ Cof<float> cof_at(const float *cof, size_t n, unsigned o)
 {
     Cof<float> a;
@@ -1445,8 +1452,8 @@ cudaError_t linear_sweep(int N, double h, float *e, const float *f, const float 
     const size_t n = (size_t)N * N * N;
     float *cof = work + n;
     if (!lin_fused(N, e, work)) {
-        note_launch();
-        k_cof6f<<<row_grid(N), row_block(), 0, s>>>(th, N, (float)(1.0 / (h * h)), cof);
+        const cudaError_t err = cof6_split(N, h, th, cof, s);
+        if (err != cudaSuccess) return err;
     }
     return lin_sweep(N, h, e, f, cof, th, sweeps, work, s);
 }
@@ -1785,7 +1792,7 @@ cudaError_t lin_vcycle(recon_handle *H, int l, const double *fshift = nullptr, b
     const int N = H->Nl[l];
     const double h = H->hl[l];
     const float ih2 = (float)(1.0 / (h * h));
-    if (tail_ok<float>(N)) return lin_tail(H, l, raw, raw);
+    if (tail_ok<float>(N)) return lin_tail(H, l, H->e32[l], H->f32[l], H->cof32, raw, raw);
     CK(lin_sweep(N, h, H->e32[l], H->f32[l], H->cof32[l], H->t32[l], cf.nu1, H->work32, s, fshift));
     const int Nc = H->Nl[l + 1];
     const size_t nc = ncell(Nc);
@@ -1922,9 +1929,7 @@ cudaError_t mixed_correct(recon_handle *H, double *phi)
     for (int l = 1; l < H->nlev; ++l) CK(restrict_plain<float>(H->Nl[l - 1], H->t32[l - 1], H->t32[l], s));
     for (int l = 0; l < H->nlev; ++l) {
         if (H->Nl[l] >= kFusedMinN) continue;   // formed from theta32 in the kernels
-        note_launch();
-        k_cof6f<<<row_grid(H->Nl[l]), row_block(), 0, s>>>(H->t32[l], H->Nl[l],
-                                                           (float)(1.0 / (H->hl[l] * H->hl[l])), H->cof32[l]);
+        CK(cof6_split(H->Nl[l], H->hl[l], H->t32[l], H->cof32[l], s));
     }
     CK(cudaMemsetAsync(H->e32[0], 0, sizeof(float) * n, s));
     for (int v = 0; v < H->cfg.mixed_linear_vcycles; ++v)

@@ -1022,7 +1022,7 @@ cudaError_t fas_tail(recon_handle *H, int l, T *t, const T *g, const double *cpt
 template cudaError_t fas_tail<float>(recon_handle *, int, float *, const float *, const double *, bool);
 template cudaError_t fas_tail<double>(recon_handle *, int, double *, const double *, const double *, bool);
 
-cudaError_t lin_tail(recon_handle *H, int l, bool raw, bool zero)
+cudaError_t lin_tail(recon_handle *H, int l, float *e, const float *f, const float *const *cof, bool raw, bool zero)
 {
     const recon_config &cf = H->cfg;
     TailArgs<float> A{};
@@ -1033,10 +1033,10 @@ cudaError_t lin_tail(recon_handle *H, int l, bool raw, bool zero)
         const double h = H->hl[l + q];
         A.ih2[q] = (float)(1.0 / (h * h));
         A.h2_6[q] = (float)(h * h / 6.0);
-        A.cof[q] = H->cof32[l + q];
+        A.cof[q] = cof[l + q];
     }
-    A.t = H->e32[l];
-    A.g = H->f32[l];
+    A.t = e;
+    A.g = f;
     A.nu1 = cf.nu1;
     A.nu2 = cf.nu2;
     A.cmax = cf.coarse_max_sweeps;
