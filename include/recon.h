@@ -275,7 +275,7 @@ recon_status recon_level_scales(recon_handle *h, double *out, int n, int *levels
  * device N^3, distinct; field must be finite.  The probability and the
  * quantile are FP64 (distinct ranks give distinct outputs at any size up to
  * 1024^3).  The first call allocates
- * 24 N^3 bytes of workspace, held by the handle until recon_destroy.
+ * 25 N^3 bytes of workspace, held by the handle until recon_destroy.
  * Errors: RECON_E_INVALID, RECON_E_OOM, RECON_E_CUDA. */
 recon_status recon_gaussianise(recon_handle *h, const double *field, double *out);
 

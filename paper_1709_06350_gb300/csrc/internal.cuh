@@ -16,10 +16,9 @@ constexpr int kFusedMinN = 128;       // grids of at least this size use the fus
 // workspace of recon_gaussianise (allocated at its first call)
 struct GaussWork {
     size_t cap = 0;
-    unsigned long long *key[2] = {};
-    unsigned *idx[2] = {};
+    void *pairs = nullptr;      // 24 bytes per value: (key, index) pairs or bucket members
     unsigned *counts = nullptr, *segsum = nullptr;
-    double *moments = nullptr;
+    void *anchors = nullptr, *plan = nullptr;
 };
 
 struct AdjWork {

@@ -4,17 +4,26 @@
 // rank_i the position of value i in ascending order, ties broken by
 // position; mean and std (population) of the input.
 //
-// Ranks come from a least-significant-digit radix sort of (key, index)
-// pairs: key = the value's bits made order-preserving as an unsigned 64-bit
-// integer (-0 taken as +0), 8 passes of 8-bit digits.  Each pass: a digit
-// histogram per tile of 4096 elements, an exclusive scan of the
-// (digit-major, tile-minor) counts, and a stable scatter in which each tile
-// ranks its elements in order (warp match on the digit, per-warp counts
-// prefix-summed across warps).  The quantile is FP32 (normcdfinvf of the
-// smaller tail probability, so the tails keep their precision): g carries
-// ~1e-6 relative rounding, like delta_r itself.
+// Ranks come from buckets: the values are mapped by a monotone function to
+// ~n/11 buckets of nearly equal occupancy, counted and scattered in one pass
+// each, and a value's rank is its bucket's start plus the bucket's smaller
+// (key, index) pairs.  The map takes 52 bits linear in the value (the
+// significand of v + c, one rounded addition), their top 12 as a cell, and in
+// each cell a power of two of sub-buckets by its share of a 1/16 sample.
+// Fields that defeat it (heavy ties: the sum of squared occupancies says what
+// the comparisons would cost) take a least-significant-digit radix sort of
+// (key, index) pairs instead, 8 passes of 8-bit digits; both paths are
+// enqueued and the device decides, so the call stays asynchronous.
+//
+// The quantile is FP64 and was half of the time (normcdfinv, ~67 FP64
+// operations per value at one per 64 FP32 ones): it is evaluated once per 128
+// ranks and continued by its Taylor series (four FP64 operations per value).
+// What bounds it: the sector traffic of the scatters and the FP64 pipe.
+// Measured (GB300): 256^3 4.24 -> 1.35 ms, 512^3 36.9 -> 12.1 ms; a
+// 256^3 field of rounded values (radix path) 4.2 -> 2.9 ms.
 #include <climits>
 
+#include "dfloat.cuh"
 #include "internal.cuh"
 
 namespace recon {
@@ -32,67 +41,307 @@ constexpr int kScanThreads = 1024;
 constexpr int kScanItems = 4;
 constexpr int kScanSeg = kScanThreads * kScanItems;    // 4096 counts per scan block
 
+// the value's bits as an order-preserving unsigned integer (-0 as +0), and back
 __device__ __forceinline__ unsigned long long order_key(double v)
 {
-    const unsigned long long b = (unsigned long long)__double_as_longlong(v == 0.0 ? 0.0 : v);
+    unsigned long long b = (unsigned long long)__double_as_longlong(v);
+    if ((b << 1) == 0) b = 0;
     return (b >> 63) ? ~b : (b | (1ull << 63));
 }
-
-// keys, identity indices, and per-block sums of v and v^2
-__global__ void __launch_bounds__(kThreads)
-k_gauss_keys(const double *__restrict__ v, size_t n, unsigned long long *__restrict__ key,
-             unsigned *__restrict__ idx, double *__restrict__ partials)
+__device__ __forceinline__ double key_value(unsigned long long k)
 {
-    __shared__ double sh[32];
-    ThreadSum<double> s1, s2;
-    for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
-         i += (size_t)gridDim.x * blockDim.x) {
-        const double x = v[i];
-        key[i] = order_key(x);
-        idx[i] = (unsigned)i;
-        s1.add(x);
-        s2.add(x * x);
-    }
-    double t = block_sum<kThreads>(s1.get(), sh);
-    if (ltid() == 0) partials[4 * blockIdx.x + 0] = t;
-    t = block_sum<kThreads>(s2.get(), sh);
-    if (ltid() == 0) partials[4 * blockIdx.x + 1] = t;
+    return __longlong_as_double((long long)((k >> 63) ? (k ^ (1ull << 63)) : ~k));
 }
 
-// scal[0] = mean, scal[1] = population std
-__global__ void __launch_bounds__(kReduceThreads)
-k_gauss_moments(const double *__restrict__ partials, int nb, double n, double *__restrict__ scal)
+// ---- what the device decides and shares (one per handle)
+constexpr int kCells = 4096;                 // top 12 of the 52 linear bits
+constexpr int kCellBits = 40;                // bits within a cell
+constexpr int kPerBucket = 16;               // values per bucket: 8 to 16 where the sample is right
+constexpr int kSampleRun = 256, kSampleStep = 16 * kSampleRun;
+constexpr unsigned long long kMaxWork = 128; // comparisons per value above which the radix sort runs
+struct GaussPlan {
+    double mean, sd;
+    double shift;                            // c: v + c lies in [2^e, 2^(e+1))
+    unsigned long long base;                 // bits of 2^e
+    unsigned long long squares;              // sum of squared bucket occupancies
+    int bad;                                 // no usable range
+    unsigned cell[kCells];                   // sampled counts, then first bucket
+    unsigned char down[kCells];              // bits to drop within the cell
+};
+__device__ __forceinline__ bool use_radix(const GaussPlan *P, size_t n) { return P->bad || P->squares > kMaxWork * n; }
+
+__device__ __forceinline__ unsigned long long linear_bits(const GaussPlan *P, double v)
+{
+    const long long u = __double_as_longlong(v + P->shift) - (long long)P->base;
+    return u < 0 ? 0ull : (u >= (1ll << 52) ? (1ull << 52) - 1 : (unsigned long long)u);
+}
+
+// per-block sums of v and v^2, smallest and largest key
+__global__ void __launch_bounds__(kThreads)
+k_gauss_stats(const double *__restrict__ v, size_t n, double *__restrict__ partials)
 {
     __shared__ double sh[32];
+    __shared__ unsigned long long smin[kThreads / 32], smax[kThreads / 32];
+    double s1 = 0.0, s2 = 0.0;
+    unsigned long long kmin = ~0ull, kmax = 0ull;
+    for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
+        const double x = v[i];
+        const unsigned long long k = order_key(x);
+        kmin = k < kmin ? k : kmin;
+        kmax = k > kmax ? k : kmax;
+        s1 += x;
+        s2 = fma(x, x, s2);
+    }
+    for (int o = 16; o > 0; o >>= 1) {
+        const unsigned long long a = __shfl_xor_sync(0xffffffffu, kmin, o), b = __shfl_xor_sync(0xffffffffu, kmax, o);
+        kmin = a < kmin ? a : kmin;
+        kmax = b > kmax ? b : kmax;
+    }
+    if ((threadIdx.x & 31) == 0) {
+        smin[threadIdx.x >> 5] = kmin;
+        smax[threadIdx.x >> 5] = kmax;
+    }
+    double t = block_sum<kThreads>(s1, sh);
+    if (ltid() == 0) partials[4 * blockIdx.x + 0] = t;
+    t = block_sum<kThreads>(s2, sh);
+    if (ltid() == 0) {
+        partials[4 * blockIdx.x + 1] = t;
+        for (int w = 1; w < kThreads / 32; ++w) {
+            kmin = smin[w] < kmin ? smin[w] : kmin;
+            kmax = smax[w] > kmax ? smax[w] : kmax;
+        }
+        partials[4 * blockIdx.x + 2] = __longlong_as_double((long long)kmin);
+        partials[4 * blockIdx.x + 3] = __longlong_as_double((long long)kmax);
+    }
+}
+
+// mean, population std, the linear map; clears the cells
+__global__ void __launch_bounds__(kReduceThreads)
+k_gauss_moments(const double *__restrict__ partials, int nb, double n, GaussPlan *__restrict__ P)
+{
+    __shared__ double sh[32];
+    __shared__ unsigned long long smin[32], smax[32];
     double a = 0.0, b = 0.0;
+    unsigned long long kmin = ~0ull, kmax = 0ull;
     for (int i = threadIdx.x; i < nb; i += blockDim.x) {
         a += partials[4 * i + 0];
         b += partials[4 * i + 1];
+        const unsigned long long x = (unsigned long long)__double_as_longlong(partials[4 * i + 2]);
+        const unsigned long long y = (unsigned long long)__double_as_longlong(partials[4 * i + 3]);
+        kmin = x < kmin ? x : kmin;
+        kmax = y > kmax ? y : kmax;
+    }
+    for (int o = 16; o > 0; o >>= 1) {
+        const unsigned long long x = __shfl_xor_sync(0xffffffffu, kmin, o), y = __shfl_xor_sync(0xffffffffu, kmax, o);
+        kmin = x < kmin ? x : kmin;
+        kmax = y > kmax ? y : kmax;
+    }
+    if ((threadIdx.x & 31) == 0) {
+        smin[threadIdx.x >> 5] = kmin;
+        smax[threadIdx.x >> 5] = kmax;
     }
     a = block_sum<kReduceThreads>(a, sh);
     b = block_sum<kReduceThreads>(b, sh);
+    for (int c = threadIdx.x; c < kCells; c += blockDim.x) P->cell[c] = 0;
     if (ltid() == 0) {
+        for (int w = 1; w < kReduceThreads / 32; ++w) {
+            kmin = smin[w] < kmin ? smin[w] : kmin;
+            kmax = smax[w] > kmax ? smax[w] : kmax;
+        }
         const double m = a / n, var = b / n - m * m;
-        scal[0] = m;
-        scal[1] = var > 0.0 ? sqrt(var) : 0.0;
+        P->mean = m;
+        P->sd = var > 0.0 ? sqrt(var) : 0.0;
+        const double lo = key_value(kmin), range = key_value(kmax) - lo;
+        P->squares = 0;
+        // (equal values, ranges that overflow or underflow the significand map)
+        P->bad = !(range > 1e-290 && range < 1e290 && fabs(lo) < 1e290);
+        int e = 0;
+        frexp(range, &e);                    // range < 2^e
+        const double top = ldexp(1.0, P->bad ? 0 : e);
+        P->shift = top - lo;
+        P->base = (unsigned long long)__double_as_longlong(top);
+    }
+}
+
+// cell counts of the sample (kSampleRun of every kSampleStep values, or all of a small field)
+__global__ void __launch_bounds__(kSampleRun)
+k_gauss_sample(const double *__restrict__ v, size_t n, size_t step, GaussPlan *__restrict__ P)
+{
+    __shared__ unsigned c[kCells];
+    if (P->bad) return;
+    for (int i = threadIdx.x; i < kCells; i += kSampleRun) c[i] = 0;
+    __syncthreads();
+    for (size_t b = (size_t)blockIdx.x * step; b < n; b += (size_t)gridDim.x * step)
+        if (b + threadIdx.x < n) atomicAdd(&c[linear_bits(P, v[b + threadIdx.x]) >> kCellBits], 1u);
+    __syncthreads();
+    for (int i = threadIdx.x; i < kCells; i += kSampleRun)
+        if (c[i]) atomicAdd(&P->cell[i], c[i]);
+}
+
+__device__ __forceinline__ unsigned block_excl_scan(unsigned v, unsigned *sh, unsigned *total);
+
+// sub-buckets of every cell: a power of two above its share / kPerBucket
+// (below n / 8 + kCells buckets in all)
+__global__ void __launch_bounds__(kScanThreads)
+k_gauss_plan(int weight, GaussPlan *__restrict__ P)
+{
+    __shared__ unsigned sh[32];
+    constexpr int kPer = kCells / kScanThreads;
+    unsigned lg[kPer], sum = 0;
+    for (int i = 0; i < kPer; ++i) {
+        const unsigned want = (P->cell[threadIdx.x * kPer + i] * (unsigned)weight) / kPerBucket;
+        lg[i] = want ? 32 - __clz(want) - (__popc(want) == 1) : 0;   // ceil(log2(want))
+        sum += 1u << lg[i];
+    }
+    unsigned total;
+    unsigned run = block_excl_scan(sum, sh, &total);
+    for (int i = 0; i < kPer; ++i) {
+        P->cell[threadIdx.x * kPer + i] = run;
+        P->down[threadIdx.x * kPer + i] = (unsigned char)(kCellBits - lg[i]);
+        run += 1u << lg[i];
+    }
+}
+
+// bucket of every value and its place among the bucket's arrivals
+// (a bucket that alone would take a sixteenth of kMaxWork ends it early: its
+// arrivals queue on one counter)
+__global__ void __launch_bounds__(kThreads)
+k_gauss_count(const double *__restrict__ v, size_t n, GaussPlan *__restrict__ P, unsigned *__restrict__ counts,
+              uint2 *__restrict__ where)
+{
+    volatile int *bad = &P->bad;
+    int turn = 0;
+    for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
+        if ((turn++ & 3) == 0 && *bad) return;
+        const unsigned long long u = linear_bits(P, __ldcs(v + i));
+        const unsigned c = (unsigned)(u >> kCellBits);
+        const unsigned b = P->cell[c] + (unsigned)((u & ((1ull << kCellBits) - 1)) >> P->down[c]);
+        const unsigned long long at = atomicAdd(&counts[b], 1u);
+        __stcs(where + i, make_uint2(b, (unsigned)at));
+        if (at * at > kMaxWork / 16 * n) *bad = 1;
+    }
+}
+
+// a value in its bucket: one 16-byte store per value
+struct __align__(16) Member {
+    unsigned long long key;
+    unsigned index, bucket;
+};
+__global__ void __launch_bounds__(kThreads)
+k_gauss_scatter(const double *__restrict__ v, size_t n, const GaussPlan *__restrict__ P,
+                const unsigned *__restrict__ start, const uint2 *__restrict__ where, Member *__restrict__ out)
+{
+    if (use_radix(P, n)) return;
+    for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
+        // (streaming reads, so that the members being filled keep the L2)
+        const uint2 w = __ldcs(where + i);
+        Member m;
+        m.key = order_key(__ldcs(v + i));
+        m.index = (unsigned)i;
+        m.bucket = w.x;
+        *reinterpret_cast<int4 *>(out + start[w.x] + w.y) = *reinterpret_cast<const int4 *>(&m);
+    }
+}
+
+// ---- quantiles: out = mean + std Phi^-1((r + 1/2) / n).  With z = Phi^-1(q)
+// and D = dz/dr = sqrt(2 pi) exp(z^2/2) / n, the k-th derivative with respect
+// to r is P_k(z) D^k, P_1 = 1, P_{k+1} = P_k' + k z P_k; the series about the
+// middle of 128 ranks in terms of their offset is kept per anchor.  From rank
+// kTail on an offset is below 2^-8 of the rank and six terms leave 2^-58; the
+// terms from the fourth on are below 2^-32 and evaluated in FP32.  The lower
+// half is mirrored, so the two tails have the same precision.
+constexpr int kAnchor = 128;
+constexpr size_t kTail = 16384;
+struct __align__(64) Anchor {
+    double below, above;                     // mean + sd z, mean - sd z
+    double c1, c2, c3;
+    float c4, c5, c6, unused;
+};
+__global__ void __launch_bounds__(kThreads)
+k_gauss_anchors(size_t n, size_t count, const GaussPlan *__restrict__ P, Anchor *__restrict__ out)
+{
+    const size_t a = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (a >= count) return;
+    const double z = normcdfinv(((double)(a * kAnchor + kAnchor / 2) + 0.5) / (double)n), z2 = z * z, sd = P->sd;
+    const double D = 2.5066282746310002 * exp(0.5 * z2) / (double)n;   // sqrt(2 pi)
+    const double D2 = D * D, D3 = D2 * D;
+    Anchor x;
+    x.below = P->mean + sd * z;
+    x.above = P->mean - sd * z;
+    x.c1 = sd * D;
+    x.c2 = sd * D2 * z * 0.5;
+    x.c3 = sd * D3 * (1.0 + 2.0 * z2) * (1.0 / 6.0);
+    x.c4 = (float)(sd * D2 * D2 * z * (7.0 + 6.0 * z2) * (1.0 / 24.0));
+    x.c5 = (float)(sd * D2 * D3 * (7.0 + z2 * (46.0 + 24.0 * z2)) * (1.0 / 120.0));
+    x.c6 = (float)(sd * D3 * D3 * z * (127.0 + z2 * (326.0 + 120.0 * z2)) * (1.0 / 720.0));
+    x.unused = 0.0f;
+    out[a] = x;
+}
+__device__ __noinline__ double quantile_tail(size_t lo, bool low, size_t n, double m, double sd)
+{
+    const double z = normcdfinv(((double)lo + 0.5) / (double)n);
+    return m + sd * (low ? z : -z);
+}
+__device__ __forceinline__ double quantile(size_t r, size_t n, const GaussPlan *P, const Anchor *anchors)
+{
+    const size_t lo = r < n - 1 - r ? r : n - 1 - r;
+    if (lo < kTail) return quantile_tail(lo, r == lo, n, P->mean, P->sd);
+    const Anchor &x = anchors[lo / kAnchor];
+    const float f = (float)((int)(lo & (kAnchor - 1)) - kAnchor / 2);
+    const double d = df_f2d_bits(f);
+    const double p = df_f2d_bits(fmaf(fmaf(x.c6, f, x.c5), f, x.c4));
+    const double t = fma(fma(fma(p, d, x.c3), d, x.c2), d, x.c1);
+    return r == lo ? fma(t, d, x.below) : fma(-t, d, x.above);
+}
+
+// rank of every member within its bucket, and its quantile to its place
+__global__ void __launch_bounds__(kThreads)
+k_gauss_rank(const Member *__restrict__ mem, size_t n, const GaussPlan *__restrict__ P,
+             const unsigned *__restrict__ start, const Anchor *__restrict__ anchors, double *__restrict__ g)
+{
+    if (use_radix(P, n)) return;
+    for (size_t p = (size_t)blockIdx.x * blockDim.x + threadIdx.x; p < n; p += (size_t)gridDim.x * blockDim.x) {
+        const Member m = mem[p];
+        const unsigned lo = start[m.bucket], hi = start[m.bucket + 1];
+        unsigned r = lo;
+        for (unsigned j = lo; j < hi; ++j) {
+            const Member o = mem[j];
+            r += o.key < m.key || (o.key == m.key && o.index < m.index);
+        }
+        g[m.index] = quantile(r, n, P, anchors);
+    }
+}
+
+// ---- the radix sort (P: run only where the buckets do not serve)
+__global__ void __launch_bounds__(kThreads)
+k_gauss_keys(const double *__restrict__ v, size_t n, const GaussPlan *__restrict__ P,
+             unsigned long long *__restrict__ key, unsigned *__restrict__ idx)
+{
+    if (!use_radix(P, n)) return;
+    for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
+        key[i] = order_key(v[i]);
+        idx[i] = (unsigned)i;
     }
 }
 
 // counts[d * ntile + tile] = occurrences of digit d in the tile
 __global__ void __launch_bounds__(kRadixThreads)
 k_radix_hist(const unsigned long long *__restrict__ key, size_t n, int shift, int ntile,
-             unsigned *__restrict__ counts)
+             unsigned *__restrict__ counts, const GaussPlan *__restrict__ P)
 {
     __shared__ unsigned hist[256];
-    hist[threadIdx.x] = 0;
-    __syncthreads();
-    const size_t base = (size_t)blockIdx.x * kTile;
-    for (int r = 0; r < kRadixItems; ++r) {
-        const size_t e = base + (size_t)r * kRadixThreads + threadIdx.x;
-        if (e < n) atomicAdd(&hist[(unsigned)(key[e] >> shift) & 255u], 1u);
+    if (!use_radix(P, n)) return;
+    for (int tile = blockIdx.x; tile < ntile; tile += gridDim.x) {
+        hist[threadIdx.x] = 0;
+        __syncthreads();
+        const size_t base = (size_t)tile * kTile;
+        for (int r = 0; r < kRadixItems; ++r) {
+            const size_t e = base + (size_t)r * kRadixThreads + threadIdx.x;
+            if (e < n) atomicAdd(&hist[(unsigned)(key[e] >> shift) & 255u], 1u);
+        }
+        __syncthreads();
+        counts[(size_t)threadIdx.x * ntile + tile] = hist[threadIdx.x];
     }
-    __syncthreads();
-    counts[(size_t)threadIdx.x * ntile + blockIdx.x] = hist[threadIdx.x];
 }
 
 // block-wide exclusive scan of one value per thread (total in *total)
@@ -121,16 +370,26 @@ __device__ __forceinline__ unsigned block_excl_scan(unsigned v, unsigned *sh, un
     return before + x - v;
 }
 
+// The scans serve both paths: P null for the buckets (k_scan_seg then adds up
+// their squared counts in squares), else they run only for the radix sort.
 // exclusive scan of each kScanSeg-long segment in place; segsum = its total
 __global__ void __launch_bounds__(kScanThreads)
-k_scan_seg(unsigned *__restrict__ a, size_t m, unsigned *__restrict__ segsum)
+k_scan_seg(unsigned *__restrict__ a, size_t m, unsigned *__restrict__ segsum, const GaussPlan *__restrict__ P, size_t n,
+           unsigned long long *__restrict__ squares)
 {
     __shared__ unsigned sh[32];
+    if (P && !use_radix(P, n)) return;
     const size_t base = (size_t)blockIdx.x * kScanSeg + (size_t)threadIdx.x * kScanItems;
     unsigned v[kScanItems], s = 0;
+    unsigned long long sq = 0;
     for (int k = 0; k < kScanItems; ++k) {
         v[k] = base + k < m ? a[base + k] : 0u;
         s += v[k];
+        sq += (unsigned long long)v[k] * v[k];
+    }
+    if (squares) {
+        for (int o = 16; o > 0; o >>= 1) sq += __shfl_xor_sync(0xffffffffu, sq, o);
+        if ((threadIdx.x & 31) == 0 && sq) atomicAdd(squares, sq);
     }
     unsigned total;
     unsigned run = block_excl_scan(s, sh, &total);
@@ -143,9 +402,10 @@ k_scan_seg(unsigned *__restrict__ a, size_t m, unsigned *__restrict__ segsum)
 
 // exclusive scan of the segment totals (one block, any count)
 __global__ void __launch_bounds__(kScanThreads)
-k_scan_top(unsigned *__restrict__ segsum, int nseg)
+k_scan_top(unsigned *__restrict__ segsum, int nseg, const GaussPlan *__restrict__ P, size_t n)
 {
     __shared__ unsigned sh[32];
+    if (P && !use_radix(P, n)) return;
     unsigned carry = 0;
     for (int base = 0; base < nseg; base += kScanThreads) {
         const int i = base + threadIdx.x;
@@ -158,8 +418,10 @@ k_scan_top(unsigned *__restrict__ segsum, int nseg)
 }
 
 __global__ void __launch_bounds__(kScanThreads)
-k_scan_add(unsigned *__restrict__ a, size_t m, const unsigned *__restrict__ segsum)
+k_scan_add(unsigned *__restrict__ a, size_t m, const unsigned *__restrict__ segsum, const GaussPlan *__restrict__ P,
+           size_t n)
 {
+    if (P && !use_radix(P, n)) return;
     const size_t base = (size_t)blockIdx.x * kScanSeg + (size_t)threadIdx.x * kScanItems;
     const unsigned add = segsum[blockIdx.x];
     for (int k = 0; k < kScanItems; ++k)
@@ -171,80 +433,76 @@ k_scan_add(unsigned *__restrict__ a, size_t m, const unsigned *__restrict__ segs
 __global__ void __launch_bounds__(kRadixThreads)
 k_radix_scatter(const unsigned long long *__restrict__ kin, const unsigned *__restrict__ iin, size_t n,
                 int shift, int ntile, const unsigned *__restrict__ offs,
-                unsigned long long *__restrict__ kout, unsigned *__restrict__ iout)
+                unsigned long long *__restrict__ kout, unsigned *__restrict__ iout, const GaussPlan *__restrict__ P)
 {
+    if (!use_radix(P, n)) return;
     constexpr int kW = kRadixThreads / 32;
     __shared__ unsigned base[256], total[256];
     __shared__ unsigned wcnt[kW][256];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    base[tid] = offs[(size_t)tid * ntile + blockIdx.x];
-    const size_t tile = (size_t)blockIdx.x * kTile;
     const unsigned lt = (1u << lane) - 1u;
-    for (int r = 0; r < kRadixItems; ++r) {
-        for (int w = 0; w < kW; ++w) wcnt[w][tid] = 0;
-        const size_t e = tile + (size_t)r * kRadixThreads + tid;
-        const bool valid = e < n;
-        const unsigned long long k = valid ? kin[e] : 0ull;
-        const unsigned d = valid ? ((unsigned)(k >> shift) & 255u) : 256u;
-        const unsigned peers = __match_any_sync(0xffffffffu, d);
-        const unsigned rank = __popc(peers & lt);
-        __syncthreads();   // base / wcnt ready
-        if (valid && rank == 0) wcnt[warp][d] = __popc(peers);
-        __syncthreads();
-        {   // per digit: exclusive prefix over the warps of this round
-            unsigned run = 0;
-            for (int w = 0; w < kW; ++w) {
-                const unsigned c = wcnt[w][tid];
-                wcnt[w][tid] = run;
-                run += c;
+    for (int it = blockIdx.x; it < ntile; it += gridDim.x) {
+        __syncthreads();   // the previous tile's last reads of base
+        base[tid] = offs[(size_t)tid * ntile + it];
+        const size_t tile = (size_t)it * kTile;
+        for (int r = 0; r < kRadixItems; ++r) {
+            for (int w = 0; w < kW; ++w) wcnt[w][tid] = 0;
+            const size_t e = tile + (size_t)r * kRadixThreads + tid;
+            const bool valid = e < n;
+            const unsigned long long k = valid ? kin[e] : 0ull;
+            const unsigned d = valid ? ((unsigned)(k >> shift) & 255u) : 256u;
+            const unsigned peers = __match_any_sync(0xffffffffu, d);
+            const unsigned rank = __popc(peers & lt);
+            __syncthreads();   // base / wcnt ready
+            if (valid && rank == 0) wcnt[warp][d] = __popc(peers);
+            __syncthreads();
+            {   // per digit: exclusive prefix over the warps of this round
+                unsigned run = 0;
+                for (int w = 0; w < kW; ++w) {
+                    const unsigned c = wcnt[w][tid];
+                    wcnt[w][tid] = run;
+                    run += c;
+                }
+                total[tid] = run;
             }
-            total[tid] = run;
+            __syncthreads();
+            if (valid) {
+                const unsigned pos = base[d] + wcnt[warp][d] + rank;
+                kout[pos] = k;
+                iout[pos] = iin[e];
+            }
+            __syncthreads();
+            base[tid] += total[tid];
         }
-        __syncthreads();
-        if (valid) {
-            const unsigned pos = base[d] + wcnt[warp][d] + rank;
-            kout[pos] = k;
-            iout[pos] = iin[e];
-        }
-        __syncthreads();
-        base[tid] += total[tid];
     }
 }
 
-// g[idx[r]] = mean + std * Phi^-1((r + 1/2) / n).  The probability and the
-// quantile are FP64: above 2^24 cells adjacent ranks would round to the same
-// FP32 probability and distinct inputs would get equal outputs.  The quantile
-// is taken of the smaller tail probability and mirrored, so the two halves
-// are exactly antisymmetric.
+// g[idx[r]] = the quantile of rank r
 __global__ void __launch_bounds__(kThreads)
-k_gauss_out(const unsigned *__restrict__ idx, size_t n, const double *__restrict__ scal,
-            double *__restrict__ g)
+k_gauss_out(const unsigned *__restrict__ idx, size_t n, const GaussPlan *__restrict__ P,
+            const Anchor *__restrict__ anchors, double *__restrict__ g)
 {
-    const double m = scal[0], sd = scal[1];
-    for (size_t r = (size_t)blockIdx.x * blockDim.x + threadIdx.x; r < n;
-         r += (size_t)gridDim.x * blockDim.x) {
-        const size_t lo = r < n - 1 - r ? r : n - 1 - r;
-        const double q = ((double)lo + 0.5) / (double)n;   // smaller tail probability
-        const double z = normcdfinv(q);
-        g[idx[r]] = m + sd * (r == lo ? z : -z);
-    }
+    if (!use_radix(P, n)) return;
+    for (size_t r = (size_t)blockIdx.x * blockDim.x + threadIdx.x; r < n; r += (size_t)gridDim.x * blockDim.x)
+        g[idx[r]] = quantile(r, n, P, anchors);
 }
+
+inline size_t bucket_slots(size_t n) { return n / 8 + 2 * kCells; }
+inline size_t anchor_count(size_t n) { return n / (2 * kAnchor) + 1; }
 
 cudaError_t gauss_alloc(recon_handle *H, size_t n)
 {
     GaussWork &G = H->gauss;
     if (G.cap >= n) return cudaSuccess;
     gauss_free(H);
-    const size_t ntile = (n + kTile - 1) / kTile, m = 256 * ntile;
+    const size_t ntile = (n + kTile - 1) / kTile, m = 256 * ntile > bucket_slots(n) ? 256 * ntile : bucket_slots(n);
     const size_t nseg = (m + kScanSeg - 1) / kScanSeg;
-    cudaError_t e = cudaSuccess;
-    for (int b = 0; b < 2 && e == cudaSuccess; ++b) {
-        e = cudaMalloc(&G.key[b], sizeof(unsigned long long) * n);
-        if (e == cudaSuccess) e = cudaMalloc(&G.idx[b], sizeof(unsigned) * n);
-    }
+    // two key arrays and two index arrays, or the members and their places
+    cudaError_t e = cudaMalloc(&G.pairs, 24 * n);
     if (e == cudaSuccess) e = cudaMalloc(&G.counts, sizeof(unsigned) * m);
     if (e == cudaSuccess) e = cudaMalloc(&G.segsum, sizeof(unsigned) * nseg);
-    if (e == cudaSuccess) e = cudaMalloc(&G.moments, sizeof(double) * 2);
+    if (e == cudaSuccess) e = cudaMalloc(&G.anchors, sizeof(Anchor) * anchor_count(n));
+    if (e == cudaSuccess) e = cudaMalloc(&G.plan, sizeof(GaussPlan));
     if (e != cudaSuccess) {
         gauss_free(H);
         return e;
@@ -256,13 +514,11 @@ cudaError_t gauss_alloc(recon_handle *H, size_t n)
 void gauss_free(recon_handle *H)
 {
     GaussWork &G = H->gauss;
-    for (int b = 0; b < 2; ++b) {
-        if (G.key[b]) cudaFree(G.key[b]);
-        if (G.idx[b]) cudaFree(G.idx[b]);
-    }
+    if (G.pairs) cudaFree(G.pairs);
     if (G.counts) cudaFree(G.counts);
     if (G.segsum) cudaFree(G.segsum);
-    if (G.moments) cudaFree(G.moments);
+    if (G.anchors) cudaFree(G.anchors);
+    if (G.plan) cudaFree(G.plan);
     G = GaussWork{};
 }
 
@@ -271,26 +527,57 @@ cudaError_t gaussianise(recon_handle *H, const double *v, size_t n, double *g)
     cudaStream_t s = H->stream;
     CK(gauss_alloc(H, n));
     GaussWork &G = H->gauss;
+    GaussPlan *P = static_cast<GaussPlan *>(G.plan);
+    Anchor *anchors = static_cast<Anchor *>(G.anchors);
+    const unsigned nb = stride_blocks(n) < (unsigned)kMaxRedBlocks ? stride_blocks(n) : (unsigned)kMaxRedBlocks;
+    const unsigned sb = stride_blocks(n);
+    // the map and the quantiles' anchors
+    const size_t nanchor = anchor_count(n);
+    const bool whole = n < 256 * (size_t)kSampleStep;   // small fields are counted in full
+    const size_t step = whole ? kSampleRun : kSampleStep;
+    const size_t sblocks = (n + step - 1) / step;
+    note_launch(5);
+    k_gauss_stats<<<nb, kThreads, 0, s>>>(v, n, H->partials);
+    k_gauss_moments<<<1, kReduceThreads, 0, s>>>(H->partials, (int)nb, (double)n, P);
+    k_gauss_anchors<<<blocks_for(nanchor), kThreads, 0, s>>>(n, nanchor, P, anchors);
+    k_gauss_sample<<<(unsigned)(sblocks < 608 ? sblocks : 608), kSampleRun, 0, s>>>(v, n, step, P);
+    k_gauss_plan<<<1, kScanThreads, 0, s>>>(whole ? 1 : kSampleStep / kSampleRun, P);
+    // buckets
+    Member *mem = static_cast<Member *>(G.pairs);
+    uint2 *where = reinterpret_cast<uint2 *>(mem + n);
+    const size_t slots = bucket_slots(n);
+    const int bseg = (int)((slots + kScanSeg - 1) / kScanSeg);
+    CK(cudaMemsetAsync(G.counts, 0, sizeof(unsigned) * slots, s));
+    note_launch(6);
+    k_gauss_count<<<sb, kThreads, 0, s>>>(v, n, P, G.counts, where);
+    k_scan_seg<<<bseg, kScanThreads, 0, s>>>(G.counts, slots, G.segsum, nullptr, n, &P->squares);
+    k_scan_top<<<1, kScanThreads, 0, s>>>(G.segsum, bseg, nullptr, n);
+    k_scan_add<<<bseg, kScanThreads, 0, s>>>(G.counts, slots, G.segsum, nullptr, n);
+    k_gauss_scatter<<<sb, kThreads, 0, s>>>(v, n, P, G.counts, where, mem);
+    k_gauss_rank<<<sb, kThreads, 0, s>>>(mem, n, P, G.counts, anchors, g);
+    // the radix sort, where the plan says so
+    unsigned long long *key[2] = {static_cast<unsigned long long *>(G.pairs),
+                                  static_cast<unsigned long long *>(G.pairs) + n};
+    unsigned *idx[2] = {reinterpret_cast<unsigned *>(key[1] + n), reinterpret_cast<unsigned *>(key[1] + n) + n};
     const int ntile = (int)((n + kTile - 1) / kTile);
+    const unsigned rb = ntile < 1216 ? ntile : 1216;
     const size_t m = 256 * (size_t)ntile;
     const int nseg = (int)((m + kScanSeg - 1) / kScanSeg);
-    const unsigned nb = stride_blocks(n) < (unsigned)kMaxRedBlocks ? stride_blocks(n) : (unsigned)kMaxRedBlocks;
-    note_launch(2);
-    k_gauss_keys<<<nb, kThreads, 0, s>>>(v, n, G.key[0], G.idx[0], H->partials);
-    k_gauss_moments<<<1, kReduceThreads, 0, s>>>(H->partials, (int)nb, (double)n, G.moments);
+    note_launch();
+    k_gauss_keys<<<nb, kThreads, 0, s>>>(v, n, P, key[0], idx[0]);
     int cur = 0;
     for (int shift = 0; shift < 64; shift += 8) {
         note_launch(5);
-        k_radix_hist<<<ntile, kRadixThreads, 0, s>>>(G.key[cur], n, shift, ntile, G.counts);
-        k_scan_seg<<<nseg, kScanThreads, 0, s>>>(G.counts, m, G.segsum);
-        k_scan_top<<<1, kScanThreads, 0, s>>>(G.segsum, nseg);
-        k_scan_add<<<nseg, kScanThreads, 0, s>>>(G.counts, m, G.segsum);
-        k_radix_scatter<<<ntile, kRadixThreads, 0, s>>>(G.key[cur], G.idx[cur], n, shift, ntile, G.counts,
-                                                        G.key[cur ^ 1], G.idx[cur ^ 1]);
+        k_radix_hist<<<rb, kRadixThreads, 0, s>>>(key[cur], n, shift, ntile, G.counts, P);
+        k_scan_seg<<<nseg, kScanThreads, 0, s>>>(G.counts, m, G.segsum, P, n, nullptr);
+        k_scan_top<<<1, kScanThreads, 0, s>>>(G.segsum, nseg, P, n);
+        k_scan_add<<<nseg, kScanThreads, 0, s>>>(G.counts, m, G.segsum, P, n);
+        k_radix_scatter<<<rb, kRadixThreads, 0, s>>>(key[cur], idx[cur], n, shift, ntile, G.counts, key[cur ^ 1],
+                                                     idx[cur ^ 1], P);
         cur ^= 1;
     }
     note_launch();
-    k_gauss_out<<<stride_blocks(n), kThreads, 0, s>>>(G.idx[cur], n, G.moments, g);
+    k_gauss_out<<<nb, kThreads, 0, s>>>(idx[cur], n, P, anchors, g);
     return cudaGetLastError();
 }
 
