@@ -127,9 +127,8 @@ __device__ __forceinline__ float2 fas_update2(const Nb19<float2> &n, float2 rhs,
 // update (the largest root, Newton-polished) with p = 9 S - 3 s^2 and
 // q = 27 det A - 9 s S + 2 s^3 - 27 rhs; that rare fallback runs behind one
 // warp vote, so the common path has no divergent branch.  Call with all lanes.
-// Fout (nullable): det A - rhs, minus the cells' residuals.
 __device__ __forceinline__ float2 fas_update2_det(const Nb19<float2> &n, float2 rhs, float ih2, float h2_2,
-                                                  float h2_6, int rule, float2 *Fout = nullptr)
+                                                  float h2_6, int rule)
 {
     const float2 axx = fma2(fma2(n.c, f2(-2.0f), add2(n.xp, n.xm)), f2(ih2), f2(1.0f));
     const float2 ayy = fma2(fma2(n.c, f2(-2.0f), add2(n.yp, n.ym)), f2(ih2), f2(1.0f));
@@ -147,7 +146,6 @@ __device__ __forceinline__ float2 fas_update2_det(const Nb19<float2> &n, float2 
     const float2 S = add2(add2(cxx, cyy), czz);
     const float2 s = add2(add2(axx, ayy), azz);
     const float2 F = sub2(det, rhs);
-    if (Fout) *Fout = F;
     const float2 tau = mul2(F, rcp2(S));
     const float2 u = mul2(tau, sub2(s, tau));
     float2 out = fma2(tau, f2(h2_2), n.c);
@@ -186,20 +184,30 @@ __device__ __forceinline__ float2 lin_update2_cof(const Cof<float2> &a, const Nb
     return fma2(mul2(r, f2(-0.5f)), rcp2(tr), e.c);
 }
 
-// det(I + H theta) of two cells
-__device__ __forceinline__ float2 det2(const Nb19<float2> &n, float ih2)
+// lin_update2 where e is 0 at the cells and all their edge neighbours: sx, sy,
+// sz the sums of their face neighbours' e (the off-diagonal cofactors drop out)
+__device__ __forceinline__ float2 lin_update2_faces(const Nb19<float2> &t, float2 sx, float2 sy, float2 sz, float2 rhs,
+                                                    float ih2, float h2)
 {
-    const float2 axx = fma2(fma2(n.c, f2(-2.0f), add2(n.xp, n.xm)), f2(ih2), f2(1.0f));
-    const float2 ayy = fma2(fma2(n.c, f2(-2.0f), add2(n.yp, n.ym)), f2(ih2), f2(1.0f));
-    const float2 azz = fma2(fma2(n.c, f2(-2.0f), add2(n.zp, n.zm)), f2(ih2), f2(1.0f));
+    const float2 axx = fma2(fma2(t.c, f2(-2.0f), add2(t.xp, t.xm)), f2(ih2), f2(1.0f));
+    const float2 ayy = fma2(fma2(t.c, f2(-2.0f), add2(t.yp, t.ym)), f2(ih2), f2(1.0f));
+    const float2 azz = fma2(fma2(t.c, f2(-2.0f), add2(t.zp, t.zm)), f2(ih2), f2(1.0f));
     const float2 q4 = f2(0.25f * ih2);
-    const float2 hxy = mul2(edge2(n.xpyp, n.xmym, n.xmyp, n.xpym), q4);
-    const float2 hyz = mul2(edge2(n.ypzp, n.ymzm, n.ymzp, n.ypzm), q4);
-    const float2 hxz = mul2(edge2(n.xpzp, n.xmzm, n.xmzp, n.xpzm), q4);
+    const float2 hxy = mul2(edge2(t.xpyp, t.xmym, t.xmyp, t.xpym), q4);
+    const float2 hyz = mul2(edge2(t.ypzp, t.ymzm, t.ymzp, t.ypzm), q4);
+    const float2 hxz = mul2(edge2(t.xpzp, t.xmzm, t.xmzp, t.xpzm), q4);
     const float2 cxx = fma2(hyz, neg2(hyz), mul2(ayy, azz));
-    const float2 cxy = fma2(hxz, hyz, neg2(mul2(hxy, azz)));
-    const float2 cxz = fma2(hxy, hyz, neg2(mul2(hxz, ayy)));
-    return fma2(axx, cxx, fma2(hxy, cxy, mul2(hxz, cxz)));
+    const float2 cyy = fma2(hxz, neg2(hxz), mul2(axx, azz));
+    const float2 czz = fma2(hxy, neg2(hxy), mul2(axx, ayy));
+    const float2 Je = fma2(czz, sz, fma2(cyy, sy, mul2(cxx, sx)));
+    const float2 tr = add2(add2(cxx, cyy), czz);
+    return mul2(fma2(Je, f2(0.5f), mul2(rhs, f2(-0.5f * h2))), rcp2(tr));
+}
+// ... and the faces too
+__device__ __forceinline__ float2 lin_update2_zero(const Nb19<float2> &t, float2 rhs, float ih2, float h2)
+{
+    const float2 z = f2(0.0f);
+    return lin_update2_faces(t, z, z, z, rhs, ih2, h2);
 }
 
 // Gauss-Seidel on J e = f for two cells (linear smoother); h2 = h^2.

@@ -82,7 +82,7 @@ inline unsigned row_grid(int N, unsigned cap = kMaxRowBlocks)
 // idle.  FP64 work pays for a warp, not for its active lanes (32^3 colour pass
 // with the 50-operation update: 9.4 us in half-full warps at 116 operations,
 // 6.8 us now).
-inline dim3 fit_block(int n) { return n > 128 ? row_block() : dim3(n, kRowX * kRowY / n, 1); }
+inline dim3 fit_block(int n) { return n > 128 || n % kRowX == 0 ? row_block() : dim3(n, kRowX * kRowY / n, 1); }
 inline unsigned fit_grid(int N, dim3 block)
 {
     const unsigned b = ((unsigned)N * (unsigned)N + block.y - 1) / block.y;
@@ -153,6 +153,63 @@ __device__ __forceinline__ double block_min(double v, double *sh)
         for (int o = 16; o > 0; o >>= 1) r = fmin(r, __shfl_down_sync(0xffffffffu, r, o));
     }
     return r;
+}
+
+// True in every thread of the block of the grid that finishes last (each
+// block calls it after thread 0 stored the block's partial results, which the
+// last block may then read); the counter is left at 0 for the next kernel.
+// Finishing a grid-wide sum in its own kernel instead of a one-block launch
+// behind it saves that launch: 5-10 us each, a tenth of a 64^3 solve.
+__device__ __forceinline__ bool last_block(unsigned *counter)
+{
+    __shared__ bool last;
+    if (ltid() == 0) {
+        __threadfence();
+        last = atomicAdd(counter, 1u) == gridDim.x - 1;
+        if (last) {
+            *counter = 0;
+            __threadfence();
+        }
+    }
+    __syncthreads();
+    return last;
+}
+
+constexpr int kMaxRedBlocks = 2048;   // grid cap of every reducing kernel
+// ... and of the ones that end in last_block: one wave of `per_sm` blocks, as a
+// block's last writes, fence and ticket take ~2 us that every further wave would
+// wait for (512^3 residual restriction: 461 us with 2048 blocks of two per SM)
+constexpr unsigned kSMs = 152;
+inline unsigned wave_grid(int N, unsigned per_sm) { return row_grid(N, kSMs * per_sm); }
+
+// Total (least) of column `col` of the blocks' partials (4 doubles each) in a
+// fixed order, in ltid() == 0 of a block of NT threads; all loads in flight at
+// once.
+template <int NT>
+__device__ __forceinline__ double total_partials(const double *partials, int nb, int col, double *sh)
+{
+    double v[kMaxRedBlocks / NT];
+#pragma unroll
+    for (int u = 0; u < kMaxRedBlocks / NT; ++u) {
+        const int b = ltid() + u * NT;
+        v[u] = b < nb ? __ldcg(partials + 4 * b + col) : 0.0;
+    }
+#pragma unroll
+    for (int u = 1; u < kMaxRedBlocks / NT; ++u) v[0] += v[u];
+    return block_sum<NT>(v[0], sh);
+}
+template <int NT>
+__device__ __forceinline__ double min_partials(const double *partials, int nb, int col, double *sh)
+{
+    double v[kMaxRedBlocks / NT];
+#pragma unroll
+    for (int u = 0; u < kMaxRedBlocks / NT; ++u) {
+        const int b = ltid() + u * NT;
+        v[u] = b < nb ? __ldcg(partials + 4 * b + col) : INFINITY;
+    }
+#pragma unroll
+    for (int u = 1; u < kMaxRedBlocks / NT; ++u) v[0] = fmin(v[0], v[u]);
+    return block_min<NT>(v[0], sh);
 }
 
 }  // namespace recon

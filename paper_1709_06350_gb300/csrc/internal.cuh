@@ -7,7 +7,7 @@
 #include "common.cuh"
 
 constexpr int kMaxLevels = 16;
-constexpr int kMaxRedBlocks = 2048;   // grid cap of every reducing kernel
+using recon::kMaxRedBlocks;
 constexpr int kFusedMinN = 128;       // grids of at least this size use the fused sweeps
 
 // Workspace of the adjoint (allocated at its first call): the potential of
@@ -55,13 +55,13 @@ struct recon_handle {
     float *t32[kMaxLevels] = {}, *g32[kMaxLevels] = {}, *told32[kMaxLevels] = {},
           *aux32[kMaxLevels] = {};
     float *e32[kMaxLevels] = {}, *f32[kMaxLevels] = {};
-    float *work32 = nullptr;
+    float *work32[kMaxLevels] = {};            // ping-pong of every level's sweeps
     float *lo32 = nullptr, *blo32 = nullptr;   // low halves of phi and b (double-float)
     float *cof32[kMaxLevels] = {};             // cofactors of I + H theta32, [6][n_l] (levels below kFusedMinN)
 
     double *scal = nullptr;      // device scalars (recon::Slot)
     double *partials = nullptr;  // kMaxRedBlocks x 4 doubles
-    int *iscratch = nullptr;     // small device ints
+    unsigned *ticket = nullptr;  // blocks done (last_block), 0 between kernels
     double *hscal = nullptr;     // pinned host mirror of scal
 
     const double *last_phi = nullptr;
@@ -95,7 +95,8 @@ int reg_sweep_chunk(int N, int want);
 // right side g + c, c from cptr or cval); chunk: planes per CTA (0 = by size)
 // gshift (nullable): a device scalar.  FAS: subtracted from every value the
 // sweep stores (a gauge shift folded into the sweep: the update depends only
-// on differences of theta).  LIN: subtracted from the right side f.
+// on differences of theta).  LIN: subtracted from the right side f.  LIN with
+// a null src: from e = 0.
 cudaError_t reg_sweep_launch(bool lin, int N, const float *src, float *dst, const float *g, const float *th,
                              const double *cptr, double cval, float ih2, float h2_6, int rule, int chunk,
                              cudaStream_t s, const double *gshift = nullptr);
@@ -110,11 +111,9 @@ cudaError_t paper_eps_planes(int N, double h, const double *theta, const double 
                              cudaStream_t s);
 
 // ---- multigrid launchers (recon_mg.cu); all asynchronous on `s`.
-// gshift (nullable): a device scalar subtracted from theta before the first
-// sweep (folded into it where the register-blocked kernel runs)
 template <typename T>
 cudaError_t sweep(int N, double h, int rule, T *t, const T *g, const double *cptr,
-                  double cval, int sweeps, T *work, cudaStream_t s, const double *gshift = nullptr);
+                  double cval, int sweeps, T *work, cudaStream_t s);
 cudaError_t residual_write(int N, double h, const double *t, const double *g,
                            const double *cptr, double cval, double *r, cudaStream_t s);
 cudaError_t det_write(int N, double h, const double *t, double *out, cudaStream_t s);

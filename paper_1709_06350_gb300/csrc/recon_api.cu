@@ -98,6 +98,7 @@ void plan(recon_handle *H, Planner &P)
             P.take(&H->g32[l], n);
             P.take(&H->e32[l], n);
             P.take(&H->f32[l], n);
+            P.take(&H->work32[l], n);
             // the fused linear sweeps form the cofactors from theta32
             if (H->Nl[l] < kFusedMinN) P.take(&H->cof32[l], 6 * n);
             if (l > 0) {
@@ -105,13 +106,12 @@ void plan(recon_handle *H, Planner &P)
                 P.take(&H->aux32[l], n);
             }
         }
-        P.take(&H->work32, n0);
         P.take(&H->lo32, n0);
         P.take(&H->blo32, n0);
     }
     P.take(&H->scal, (size_t)S_COUNT);
     P.take(&H->partials, (size_t)4 * kMaxRedBlocks);
-    P.take(&H->iscratch, (size_t)64);
+    P.take(&H->ticket, (size_t)1);
 }
 
 void free_all(recon_handle *H)
@@ -121,7 +121,6 @@ void free_all(recon_handle *H)
     };
     f(H->work64);
     f(H->work64b);
-    f(H->work32);
     f(H->lo32);
     f(H->blo32);
     for (int l = 0; l < kMaxLevels; ++l) {
@@ -137,11 +136,12 @@ void free_all(recon_handle *H)
         f(H->aux32[l]);
         f(H->e32[l]);
         f(H->f32[l]);
+        f(H->work32[l]);
         f(H->cof32[l]);
     }
     f(H->scal);
     f(H->partials);
-    f(H->iscratch);
+    f(H->ticket);
     if (H->hscal) cudaFreeHost(H->hscal);
 }
 
@@ -235,6 +235,7 @@ recon_status recon_create(int N, double L, recon_dtype dtype, recon_handle **out
     }
     cudaError_t e = prepare_kernels();
     if (e == cudaSuccess) e = cudaMemset(H->scal, 0, sizeof(double) * S_COUNT);
+    if (e == cudaSuccess) e = cudaMemset(H->ticket, 0, sizeof(unsigned));
     if (e == cudaSuccess) e = cudaDeviceSynchronize();
     if (e != cudaSuccess) {
         g_create_err = std::string("initialising the workspace: ") + cudaGetErrorString(e);

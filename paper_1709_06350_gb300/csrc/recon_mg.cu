@@ -18,6 +18,7 @@
 #include <cstdio>
 
 #include <type_traits>
+#include <utility>
 
 #include "cellmath.cuh"
 #include "cellmath2.cuh"
@@ -29,10 +30,10 @@ namespace recon {
 
 constexpr int kRowThreads = kRowX * kRowY;
 
-static inline unsigned red_blocks(size_t work, int threads = kThreads)
+static inline unsigned red_blocks(size_t work)
 {
-    size_t b = (work + threads - 1) / threads;
-    return (unsigned)(b < (size_t)kMaxRedBlocks ? (b == 0 ? 1 : b) : kMaxRedBlocks);
+    const size_t b = (work + kThreads - 1) / kThreads, most = kMaxRedBlocks;
+    return (unsigned)(b < most ? (b == 0 ? 1 : b) : most);
 }
 
 // ======================================================================
@@ -480,23 +481,24 @@ static cudaError_t fused_sweep_launch(int N, const float *src, float *dst, const
     return cudaGetLastError();
 }
 
+// Sweeps from the iterate in t with scratch w; *end (t or w) holds the result:
+// the kernels that take both colours in one pass write the other array each
+// time.
 template <typename T>
-cudaError_t sweep(int N, double h, int rule, T *t, const T *g, const double *cptr,
-                  double cval, int sweeps, T *work, cudaStream_t s, const double *gshift)
+static cudaError_t sweep_from(int N, double h, int rule, T *t, T *w, const T *g, const double *cptr, double cval,
+                              int sweeps, cudaStream_t s, const double *gshift, T **end)
 {
     const T ih2 = (T)(1.0 / (h * h)), h2_6 = (T)(h * h / 6.0);
+    *end = t;
     if constexpr (std::is_same<T, float>::value) {
-        if (sweeps > 0 && reg_sweep_ok(N, t, work, g, nullptr) && reg_sweep_ok(N, work, t, g, nullptr)) {
-            T *a = t, *b = work;
+        if (sweeps > 0 && reg_sweep_ok(N, t, w, g, nullptr) && reg_sweep_ok(N, w, t, g, nullptr)) {
             for (int it = 0; it < sweeps; ++it) {
-                const cudaError_t e = reg_sweep_launch(false, N, a, b, g, nullptr, cptr, cval, ih2, h2_6, rule,
+                const cudaError_t e = reg_sweep_launch(false, N, t, w, g, nullptr, cptr, cval, ih2, h2_6, rule,
                                                        g_fused_chunk, s, it == 0 ? gshift : nullptr);
                 if (e != cudaSuccess) return e;
-                T *tmp = a;
-                a = b;
-                b = tmp;
+                std::swap(t, w);
             }
-            if (a != t) return cudaMemcpyAsync(t, a, sizeof(T) * (size_t)N * N * N, cudaMemcpyDeviceToDevice, s);
+            *end = t;
             return cudaSuccess;
         }
     }
@@ -509,29 +511,45 @@ cudaError_t sweep(int N, double h, int rule, T *t, const T *g, const double *cpt
     // rings (measured per sweep: 128^3 209 us against 271 fused, 256^3 1.55
     // against 1.99 ms, 512^3 12.3 against 13.6 ms)
     if constexpr (std::is_same<T, float>::value) {
-        if (N >= kFusedMinN && pair_aligned(t) && pair_aligned(work)) {
-            float *a = t, *b = work;
+        if (N >= kFusedMinN && pair_aligned(t) && pair_aligned(w)) {
             for (int it = 0; it < sweeps; ++it) {
-                const cudaError_t e = fused_sweep_launch<false>(N, a, b, g, nullptr, cptr, cval, ih2, h2_6, rule, s);
+                const cudaError_t e = fused_sweep_launch<false>(N, t, w, g, nullptr, cptr, cval, ih2, h2_6, rule, s);
                 if (e != cudaSuccess) return e;
-                float *tmp = a;
-                a = b;
-                b = tmp;
+                std::swap(t, w);
             }
-            if (a != t) return cudaMemcpyAsync(t, a, sizeof(float) * (size_t)N * N * N, cudaMemcpyDeviceToDevice, s);
+            *end = t;
             return cudaSuccess;
         }
     }
     const dim3 fit = fit_block(N / 2);
     for (int it = 0; it < sweeps; ++it) {
         note_launch(2);
-        k_rb_pass<T><<<fit_grid(N, fit), fit, 0, s>>>(t, work, g, cptr, cval, N, ih2, h2_6, 0, rule);
-        k_rb_pass<T><<<fit_grid(N, fit), fit, 0, s>>>(work, t, g, cptr, cval, N, ih2, h2_6, 1, rule);
+        k_rb_pass<T><<<fit_grid(N, fit), fit, 0, s>>>(t, w, g, cptr, cval, N, ih2, h2_6, 0, rule);
+        k_rb_pass<T><<<fit_grid(N, fit), fit, 0, s>>>(w, t, g, cptr, cval, N, ih2, h2_6, 1, rule);
     }
     return cudaGetLastError();
 }
-template cudaError_t sweep<double>(int, double, int, double *, const double *, const double *, double, int, double *, cudaStream_t, const double *);
-template cudaError_t sweep<float>(int, double, int, float *, const float *, const double *, double, int, float *, cudaStream_t, const double *);
+// whether `sweeps` sweeps of a level end in the other array
+template <typename T>
+static bool sweeps_swap(int N, const T *t, const T *w, const T *g, const T *th, int sweeps)
+{
+    if constexpr (std::is_same<T, float>::value)
+        return sweeps % 2 && ((reg_sweep_ok(N, t, w, g, th) && reg_sweep_ok(N, w, t, g, th)) ||
+                              (N >= kFusedMinN && pair_aligned(t) && pair_aligned(w)));
+    return false;
+}
+
+template <typename T>
+cudaError_t sweep(int N, double h, int rule, T *t, const T *g, const double *cptr, double cval, int sweeps, T *work,
+                  cudaStream_t s)
+{
+    T *end;
+    const cudaError_t e = sweep_from<T>(N, h, rule, t, work, g, cptr, cval, sweeps, s, nullptr, &end);
+    if (e != cudaSuccess || end == t) return e;
+    return cudaMemcpyAsync(t, end, sizeof(T) * (size_t)N * N * N, cudaMemcpyDeviceToDevice, s);
+}
+template cudaError_t sweep<double>(int, double, int, double *, const double *, const double *, double, int, double *, cudaStream_t);
+template cudaError_t sweep<float>(int, double, int, float *, const float *, const double *, double, int, float *, cudaStream_t);
 
 // ======================================================================
 // residuals
@@ -557,6 +575,73 @@ k_det_write(const double *__restrict__ t, int N, double ih2, double *__restrict_
         out[offs(N, i, j, k)] = det_IH(load19<double>(t, N, i, j, k), ih2);
 }
 
+// Where the last block of a reducing kernel leaves its result: `out`
+// (S_* scalars or a slot of one level), n cells
+struct Finish {
+    unsigned *counter;
+    double n;
+    double *out;
+};
+
+// After a cycle on a level with n cells, from the partials' columns 0..2 (sums
+// of r, r^2, theta): m = mean r; c -= m; rel = sqrt(sum (r - m)^2) / denom;
+// mean theta for the gauge.  fin.out: the handle's scalars.  Out of line, so
+// that its FP64 does not disturb the register allocation of the kernels.
+template <int NT>
+__device__ __noinline__ void cycle_scalars(const double *partials, int nb, double n, double *scal)
+{
+    __shared__ double sh[3][NT / 32];
+    double p[kMaxRedBlocks / NT][3], v[3] = {0.0, 0.0, 0.0};
+#pragma unroll
+    for (int u = 0; u < kMaxRedBlocks / NT; ++u) {   // all loads in flight at once
+        const int b = ltid() + u * NT;
+        for (int x = 0; x < 3; ++x) p[u][x] = b < nb ? __ldcg(partials + 4 * b + x) : 0.0;
+    }
+#pragma unroll
+    for (int u = 0; u < kMaxRedBlocks / NT; ++u)
+        for (int x = 0; x < 3; ++x) v[x] += p[u][x];
+    for (int o = 16; o > 0; o >>= 1)
+        for (int x = 0; x < 3; ++x) v[x] += __shfl_down_sync(0xffffffffu, v[x], o);
+    if ((ltid() & 31) == 0)
+        for (int x = 0; x < 3; ++x) sh[x][ltid() >> 5] = v[x];
+    __syncthreads();
+    if (ltid() != 0) return;
+    for (int x = 0; x < 3; ++x) {
+        v[x] = 0.0;
+        for (int w = 0; w < NT / 32; ++w) v[x] += sh[x][w];
+    }
+    const double m = v[0] / n, var = v[1] - n * m * m;
+    scal[S_MEAN_R] = m;
+    scal[S_C] -= m;
+    scal[S_REL] = sqrt(var > 0.0 ? var : 0.0) / scal[S_DENOM];
+    scal[S_MEAN_T] = v[2] / n;
+}
+// ... in a launch of its own, for the kernel whose blocks last_block slows
+__global__ void __launch_bounds__(kRowThreads)
+k_finish_cycle(const double *__restrict__ partials, int nb, double n, double *__restrict__ scal)
+{
+    cycle_scalars<kRowThreads>(partials, nb, n, scal);
+}
+template <int NT>
+__device__ __forceinline__ void finish_cycle(const double *partials, const Finish &fin)
+{
+    if (last_block(fin.counter)) cycle_scalars<NT>(partials, gridDim.x, fin.n, fin.out);
+}
+
+// *fin.out = (sum of column 0) / n; no out: no mean wanted
+template <int NT>
+__device__ __noinline__ void mean_scalar(const double *partials, int nb, double n, double *out)
+{
+    __shared__ double sh[32];
+    const double s = total_partials<NT>(partials, nb, 0, sh);
+    if (ltid() == 0) *out = s / n;
+}
+template <int NT>
+__device__ __forceinline__ void finish_mean(const double *partials, const Finish &fin)
+{
+    if (fin.out && last_block(fin.counter)) mean_scalar<NT>(partials, gridDim.x, fin.n, fin.out);
+}
+
 // partials[4 b + 0..2] = sum r, sum r^2, sum theta over this block's cells,
 // r = g + c - det(I + H theta).  When f32out is set (mixed path, T = double)
 // the residual is also stored as float and theta as float in t32out.
@@ -564,7 +649,7 @@ template <typename T>
 __global__ void __launch_bounds__(kRowThreads)
 k_residual_norms(const T *__restrict__ t, const T *__restrict__ g,
                  const double *__restrict__ cptr, int N, T ih2, double *__restrict__ partials,
-                 float *__restrict__ f32out, float *__restrict__ t32out)
+                 float *__restrict__ f32out, float *__restrict__ t32out, Finish fin)
 {
     __shared__ double sh[32];
     const T c = (T)(*cptr);
@@ -588,33 +673,7 @@ k_residual_norms(const T *__restrict__ t, const T *__restrict__ g,
     if (ltid() == 0) partials[4 * blockIdx.x + 1] = v;
     v = block_sum<kRowThreads>(st.get(), sh);
     if (ltid() == 0) partials[4 * blockIdx.x + 2] = v;
-}
-
-// Single block: total of column `col` of the partials, in a fixed order.
-__device__ double sum_partials(const double *partials, int nb, int col, double *sh)
-{
-    double v = 0.0;
-    for (int b = threadIdx.x; b < nb; b += blockDim.x) v += partials[4 * b + col];
-    return block_sum<kReduceThreads>(v, sh);
-}
-
-// After a cycle on a level with n cells: m = mean r; c -= m;
-// rel = sqrt(sum (r - m)^2) / denom; mean theta for the gauge.
-__global__ void __launch_bounds__(kReduceThreads)
-k_finalize_cycle(const double *__restrict__ partials, int nb, double n, double *scal)
-{
-    __shared__ double sh[32];
-    const double sr = sum_partials(partials, nb, 0, sh);
-    const double sr2 = sum_partials(partials, nb, 1, sh);
-    const double st = sum_partials(partials, nb, 2, sh);
-    if (ltid() == 0) {
-        const double m = sr / n;
-        const double var = sr2 - n * m * m;
-        scal[S_MEAN_R] = m;
-        scal[S_C] -= m;
-        scal[S_REL] = sqrt(var > 0.0 ? var : 0.0) / scal[S_DENOM];
-        scal[S_MEAN_T] = st / n;
-    }
+    finish_cycle<kRowThreads>(partials, fin);
 }
 
 template <typename T>
@@ -709,7 +768,7 @@ template <typename T>
 __global__ void __launch_bounds__(kRowThreads, sizeof(T) == 4 ? RECON_NW_CTAS_F : RECON_WIN_CTAS)
 k_residual_norms_win(const T *__restrict__ t, const T *__restrict__ g,
                      const double *__restrict__ cptr, int N, T ih2, double *__restrict__ partials,
-                     float *__restrict__ f32out, float *__restrict__ t32out)
+                     float *__restrict__ f32out, float *__restrict__ t32out, Finish fin)
 {
     __shared__ double sh[32];
     const T c = (T)(*cptr);
@@ -748,29 +807,30 @@ k_residual_norms_win(const T *__restrict__ t, const T *__restrict__ g,
     if (ltid() == 0) partials[4 * blockIdx.x + 1] = v;
     v = block_sum<kRowThreads>(st.get(), sh);
     if (ltid() == 0) partials[4 * blockIdx.x + 2] = v;
+    finish_cycle<kRowThreads>(partials, fin);
 }
 
-// Residual norms on any grid: the windowed kernel for even N >= 32
+// Residual norms and the cycle's scalars on any grid: the windowed kernel for
+// even N >= 32
 template <typename T>
-static unsigned launch_residual_norms(const T *t, const T *g, const double *cptr, int N, T ih2,
-                                      double *partials, float *f32out, float *t32out, cudaStream_t s)
+static cudaError_t residual_norms(recon_handle *H, const T *t, const T *g, int N, T ih2, float *f32out, float *t32out)
 {
+    const Finish fin = {H->ticket, (double)N * N * N, H->scal};
     note_launch();
-    if (N % 2 == 0 && N >= 32) {
-        const unsigned nbr = row_grid(N / 2, kMaxRedBlocks);
-        k_residual_norms_win<T><<<nbr, row_block(), 0, s>>>(t, g, cptr, N, ih2, partials, f32out, t32out);
-        return nbr;
-    }
-    const unsigned nbr = row_grid(N, kMaxRedBlocks);
-    k_residual_norms<T><<<nbr, row_block(), 0, s>>>(t, g, cptr, N, ih2, partials, f32out, t32out);
-    return nbr;
+    if (N % 2 == 0 && N >= 32)
+        k_residual_norms_win<T><<<wave_grid(N / 2, 2), row_block(), 0, H->stream>>>(
+            t, g, H->scal + S_C, N, ih2, H->partials, f32out, t32out, fin);
+    else
+        k_residual_norms<T><<<wave_grid(N, 4), row_block(), 0, H->stream>>>(
+            t, g, H->scal + S_C, N, ih2, H->partials, f32out, t32out, fin);
+    return cudaGetLastError();
 }
 
 template <typename T>
 __global__ void __launch_bounds__(kRowThreads, sizeof(T) == 4 ? RECON_RR_CTAS_F : RECON_WIN_CTAS)
 k_restrict_residual(const T *__restrict__ t, const T *__restrict__ g,
                     const double *__restrict__ cptr, int Nf, T ih2, T *__restrict__ tH,
-                    T *__restrict__ toldH, T *__restrict__ rrH, double *__restrict__ partials)
+                    T *__restrict__ toldH, T *__restrict__ rrH, double *__restrict__ partials, Finish fin)
 {
     __shared__ double sh[32];
     const int Nc = Nf >> 1;
@@ -808,16 +868,10 @@ k_restrict_residual(const T *__restrict__ t, const T *__restrict__ g,
         rrH[id] = vr;
         srr.add(vr);
     }
+    if (!fin.out) return;   // a tail below takes the sum itself
     const double v = block_sum<kRowThreads>(srr.get(), sh);
     if (ltid() == 0) partials[4 * blockIdx.x + 0] = v;
-}
-
-__global__ void __launch_bounds__(kReduceThreads)
-k_finalize_mean(const double *__restrict__ partials, int nb, double n, double *out)
-{
-    __shared__ double sh[32];
-    const double s = sum_partials(partials, nb, 0, sh);
-    if (ltid() == 0) *out = s / n;
+    finish_mean<kRowThreads>(partials, fin);
 }
 
 template <typename T>
@@ -845,14 +899,74 @@ cudaError_t restrict_plain(int Nf, const T *fine, T *coarse, cudaStream_t s)
 template cudaError_t restrict_plain<double>(int, const double *, double *, cudaStream_t);
 template cudaError_t restrict_plain<float>(int, const float *, float *, cudaStream_t);
 
+// Plain restriction to several levels at once: a CTA takes a tile of 2^m cells
+// a side (m <= 4 levels, the sums of eight as in k_restrict_plain, level by
+// level in shared memory).  One launch instead of m where each would be a few
+// microseconds of latency.
+template <typename T>
+struct LevelOuts {
+    T *p[4];
+};
+template <typename T>
+__global__ void __launch_bounds__(512)
+k_restrict_tile(const T *__restrict__ f, int Nf, int m, LevelOuts<T> out)
+{
+    __shared__ T sh[2][512];
+    int side = (1 << m) >> 1;                  // cells a side of the tile on the level being made
+    int N = Nf >> 1;
+    for (int l = 0; l < m; ++l, side >>= 1, N >>= 1) {
+        const T *src = sh[(l + 1) & 1];
+        T *dst = sh[l & 1];
+        const int ss = 2 * side;
+        for (int id = threadIdx.x; id < side * side * side; id += blockDim.x) {
+            const int K = id & (side - 1), J = (id / side) & (side - 1), I = id / (side * side);
+            const int gi = blockIdx.z * side + I, gj = blockIdx.y * side + J, gk = blockIdx.x * side + K;
+            T acc = T(0);
+            for (int a = 0; a < 2; ++a)
+                for (int b = 0; b < 2; ++b)
+                    for (int c = 0; c < 2; ++c)
+                        acc += l == 0 ? f[offs(Nf, 2 * gi + a, 2 * gj + b, 2 * gk + c)]
+                                      : src[((2 * I + a) * ss + 2 * J + b) * ss + 2 * K + c];
+            acc *= T(0.125);
+            dst[id] = acc;
+            out.p[l][offs(N, gi, gj, gk)] = acc;
+        }
+        __syncthreads();
+    }
+}
+
+// arr[1 ..] = the restrictions of arr[0] (all levels).  Levels above 128^3 go
+// one by one (coalesced rows, bandwidth bound).
+template <typename T>
+cudaError_t restrict_levels(const int *Nl, int nlev, T *const *arr, cudaStream_t s)
+{
+    int l = 0;
+    while (l + 1 < nlev) {
+        if (Nl[l] > 128) {
+            const cudaError_t e = restrict_plain<T>(Nl[l], arr[l], arr[l + 1], s);
+            if (e != cudaSuccess) return e;
+            ++l;
+            continue;
+        }
+        const int m = nlev - 1 - l < 4 ? nlev - 1 - l : 4, tiles = Nl[l] >> m;
+        LevelOuts<T> out{};
+        for (int q = 0; q < m; ++q) out.p[q] = arr[l + 1 + q];
+        note_launch();
+        k_restrict_tile<T><<<dim3(tiles, tiles, tiles), m >= 4 ? 512 : 64, 0, s>>>(arr[l], Nl[l], m, out);
+        l += m;
+    }
+    return cudaGetLastError();
+}
+
 // Coarse right side, first half: rr = R r - mean(R r) (stored back in gH),
-// dH = det_H(I + H theta_H) (stored in aux), and the block minimum of the
-// scaled-defect ratio floor * max(dH, 0) / (-rr) over cells with rr < 0.
+// dH = det_H(I + H theta_H) (stored in aux), and from the minimum of the
+// scaled-defect ratio floor * max(dH, 0) / (-rr) over cells with rr < 0 the
+// level's factor s and 1 / s.
 template <typename T>
 __global__ void __launch_bounds__(kRowThreads)
 k_coarse_rhs(const T *__restrict__ tH, T *__restrict__ gH, T *__restrict__ dH,
              const double *__restrict__ mean_ptr, int Nc, T ih2, double floor_,
-             double *__restrict__ partials)
+             double *__restrict__ partials, Finish fin)
 {
     __shared__ double sh[32];
     const T m = (T)(*mean_ptr);
@@ -870,24 +984,16 @@ k_coarse_rhs(const T *__restrict__ tH, T *__restrict__ gH, T *__restrict__ dH,
             mn = cand < mn ? cand : mn;
         }
     }
-    const double v = block_min<kRowThreads>((double)mn, sh);
+    double v = block_min<kRowThreads>((double)mn, sh);
     if (ltid() == 0) partials[4 * blockIdx.x + 3] = v;
-}
-
-// s = min(1, min ratio) (1 when the safeguard is off); s < 1e-3 -> 0 (skip).
-__global__ void __launch_bounds__(kReduceThreads)
-k_finalize_scale(const double *__restrict__ partials, int nb, double floor_, double *sslot,
-                 double *pslot)
-{
-    __shared__ double sh[32];
-    double v = INFINITY;
-    for (int b = threadIdx.x; b < nb; b += blockDim.x) v = fmin(v, partials[4 * b + 3]);
-    v = block_min<kReduceThreads>(v, sh);
+    // s = min(1, min ratio) (1 when the safeguard is off); s < 1e-3 -> 0 (skip)
+    if (!last_block(fin.counter)) return;
+    v = min_partials<kRowThreads>(partials, gridDim.x, 3, sh);
     if (ltid() == 0) {
         double s = floor_ <= 0.0 ? 1.0 : fmin(1.0, v);
         if (s < 1e-3) s = 0.0;
-        *sslot = s;
-        *pslot = s > 0.0 ? 1.0 / s : 0.0;
+        fin.out[0] = s;                        // slot_scale
+        fin.out[1] = s > 0.0 ? 1.0 / s : 0.0;  // slot_pscale
     }
 }
 
@@ -902,7 +1008,7 @@ k_form_rhs(T *__restrict__ gH, const T *__restrict__ dH, size_t nc,
         gH[id] = dH[id] + sc * gH[id];
 }
 
-// fine += scale * P(cnew - cold), P cell-centred trilinear: per axis the
+// out = fine + scale * P(cnew - cold) (out may be fine), P cell-centred trilinear: per axis the
 // parent weighs 3/4 and the coarse neighbour on the fine cell's side 1/4.
 // scale = *pscale when pscale is given (0 = no correction), else `scale`.
 // A thread takes one coarse cell (threads along K, rows (I, J) grid-stride)
@@ -925,15 +1031,17 @@ struct Vec2<double> {
 template <typename T>
 __global__ void __launch_bounds__(kRowThreads)
 k_prolong_add(const T *__restrict__ cnew, const T *__restrict__ cold, int Nc,
-              const double *__restrict__ pscale, double scale, T *__restrict__ fine, int pairs)
+              const double *__restrict__ pscale, double scale, const T *fine, T *out, int pairs)
 {
     using V2 = typename Vec2<T>::type;
     const double sc = pscale ? *pscale : scale;
-    if (sc == 0.0) return;
-    // per axis the weights 3/4, 1/4 as 3 a + b, all three quarters in the scale
-    // (exact): one operation per interpolated value, which is what the FP64
-    // form waits for (FP64 128^3: 69 -> 41 us)
-    const T s = (T)(sc * (1.0 / 64.0));
+    if (sc == 0.0 && fine == out) return;
+    // FP64: per axis the weights 3/4, 1/4 as 3 a + b, all three quarters in the
+    // scale (exact): one operation per interpolated value, which is what it
+    // waits for (128^3: 69 -> 41 us)
+    constexpr bool kThree = sizeof(T) == 8;
+    const T s = (T)(kThree ? sc * (1.0 / 64.0) : sc), w0 = T(0.75), w1 = T(0.25);
+    auto mix = [&](T near, T far) { return kThree ? fma(T(3), near, far) : w0 * near + w1 * far; };
     const int Nf = 2 * Nc;
     FOR_ROWS(Nc, I, J)
     {
@@ -972,20 +1080,22 @@ k_prolong_add(const T *__restrict__ cnew, const T *__restrict__ cold, int Nc,
 #pragma unroll
                 for (int b = 0; b < 3; ++b)
 #pragma unroll
-                    for (int c = 0; c < 3; ++c) u[b][c] = fma(T(3), d[1][b][c], d[ei ? 2 : 0][b][c]);
+                    for (int c = 0; c < 3; ++c) u[b][c] = mix(d[1][b][c], d[ei ? 2 : 0][b][c]);
 #pragma unroll
                 for (int ej = 0; ej < 2; ++ej) {
                     T v[3];
 #pragma unroll
-                    for (int c = 0; c < 3; ++c) v[c] = fma(T(3), u[1][c], u[ej ? 2 : 0][c]);
+                    for (int c = 0; c < 3; ++c) v[c] = mix(u[1][c], u[ej ? 2 : 0][c]);
                     V2 x = fv[ei][ej];
-                    x.x = fma(s, fma(T(3), v[1], v[0]), x.x);
-                    x.y = fma(s, fma(T(3), v[1], v[2]), x.y);
+                    if (sc != 0.0) {   // else a skipped correction, which may hold anything
+                        x.x += s * mix(v[1], v[0]);
+                        x.y += s * mix(v[1], v[2]);
+                    }
                     if (pairs) {
-                        *reinterpret_cast<V2 *>(fine + fo[ei][ej]) = x;
+                        *reinterpret_cast<V2 *>(out + fo[ei][ej]) = x;
                     } else {
-                        fine[fo[ei][ej]] = x.x;
-                        fine[fo[ei][ej] + 1] = x.y;
+                        out[fo[ei][ej]] = x.x;
+                        out[fo[ei][ej] + 1] = x.y;
                     }
                 }
             }
@@ -994,14 +1104,20 @@ k_prolong_add(const T *__restrict__ cnew, const T *__restrict__ cold, int Nc,
 }
 
 template <typename T>
-cudaError_t prolong_add(int Nc, const T *cnew, const T *cold, const double *pscale,
-                        double scale, T *fine, cudaStream_t s)
+static cudaError_t prolong_to(int Nc, const T *cnew, const T *cold, const double *pscale, double scale, const T *fine,
+                              T *out, cudaStream_t s)
 {
     note_launch();
-    const int pairs = ((uintptr_t)fine % (2 * sizeof(T))) == 0;
+    const int pairs = (((uintptr_t)fine | (uintptr_t)out) % (2 * sizeof(T))) == 0;
     const dim3 fit = fit_block(Nc);
-    k_prolong_add<T><<<fit_grid(Nc, fit), fit, 0, s>>>(cnew, cold, Nc, pscale, scale, fine, pairs);
+    k_prolong_add<T><<<fit_grid(Nc, fit), fit, 0, s>>>(cnew, cold, Nc, pscale, scale, fine, out, pairs);
     return cudaGetLastError();
+}
+template <typename T>
+cudaError_t prolong_add(int Nc, const T *cnew, const T *cold, const double *pscale, double scale, T *fine,
+                        cudaStream_t s)
+{
+    return prolong_to<T>(Nc, cnew, cold, pscale, scale, fine, fine, s);
 }
 template cudaError_t prolong_add<double>(int, const double *, const double *, const double *, double, double *, cudaStream_t);
 template cudaError_t prolong_add<float>(int, const float *, const float *, const double *, double, float *, cudaStream_t);
@@ -1164,7 +1280,7 @@ cudaError_t det_write(int N, double h, const double *t, double *out, cudaStream_
 // domain check of b and the stop-rule denominator ||b - 1||_2
 // ======================================================================
 __global__ void __launch_bounds__(kThreads)
-k_b_stats(const double *__restrict__ b, size_t n, double *__restrict__ partials)
+k_b_stats(const double *__restrict__ b, size_t n, double *__restrict__ partials, Finish fin)
 {
     // finiteness and the minimum on the bit patterns (integer pipes); the
     // norm from the FP64 difference b - 1 widened once per thread.
@@ -1193,21 +1309,14 @@ k_b_stats(const double *__restrict__ b, size_t n, double *__restrict__ partials)
                                         : __longlong_as_double(kmin < 0 ? (kmin ^ LLONG_MAX) : kmin);
     v = block_min<kThreads>(mn, sh);
     if (ltid() == 0) partials[4 * blockIdx.x + 3] = v;
-}
-
-__global__ void __launch_bounds__(kReduceThreads)
-k_finalize_b(const double *__restrict__ partials, int nb, double *scal)
-{
-    __shared__ double sh[32];
-    const double s2 = sum_partials(partials, nb, 0, sh);
-    const double bad = sum_partials(partials, nb, 1, sh);
-    double mn = INFINITY;
-    for (int b = threadIdx.x; b < nb; b += blockDim.x) mn = fmin(mn, partials[4 * b + 3]);
-    mn = block_min<kReduceThreads>(mn, sh);
+    if (!last_block(fin.counter)) return;
+    const double t2 = total_partials<kThreads>(partials, gridDim.x, 0, sh);
+    const double tbad = total_partials<kThreads>(partials, gridDim.x, 1, sh);
+    const double tmin = min_partials<kThreads>(partials, gridDim.x, 3, sh);
     if (ltid() == 0) {
-        scal[S_DENOM] = s2 > 0.0 ? sqrt(s2) : 1.0;
-        scal[S_BBAD] = bad;
-        scal[S_BMIN] = mn;
+        fin.out[S_DENOM] = t2 > 0.0 ? sqrt(t2) : 1.0;
+        fin.out[S_BBAD] = tbad;
+        fin.out[S_BMIN] = tmin;
     }
 }
 
@@ -1307,7 +1416,8 @@ k_update_df(float *__restrict__ hi, float *__restrict__ lo, const float *__restr
 
 // block partial sums of phi_hi + phi_lo (double-float sums per thread)
 __global__ void __launch_bounds__(kThreads)
-k_df_sum(const float *__restrict__ hi, const float *__restrict__ lo, size_t n, double *__restrict__ partials)
+k_df_sum(const float *__restrict__ hi, const float *__restrict__ lo, size_t n, double *__restrict__ partials,
+         Finish fin)
 {
     __shared__ double sh[32];
     df s = df_make(0.0f, 0.0f);
@@ -1316,6 +1426,7 @@ k_df_sum(const float *__restrict__ hi, const float *__restrict__ lo, size_t n, d
         s = df_add(s, df_make(hi[id], lo[id]));
     const double v = block_sum<kThreads>(df_to_double_bits(s), sh);
     if (ltid() == 0) partials[4 * blockIdx.x + 0] = v;
+    finish_mean<kThreads>(partials, fin);
 }
 
 // phi = (phi_hi + phi_lo) - mean in FP64: the difference in double-float,
@@ -1335,27 +1446,55 @@ k_df_to_double_gauged(const float *__restrict__ hi, const float *__restrict__ lo
 // cofactors from theta inside each kernel; the coarser grids read six
 // cofactor arrays ([6][N^3]) computed once per correction (k_cof6f), stored
 // colour-split within each row (cof_slot).
+struct CofLevels {
+    int n;
+    int N[kMaxLevels];
+    unsigned block[kMaxLevels + 1];   // first block of each level
+    float ih2[kMaxLevels];
+    const float *th[kMaxLevels];
+    float *cof[kMaxLevels];
+};
+// (of several levels: each has its own range of blocks)
 __global__ void __launch_bounds__(kRowThreads)
-k_cof6f(const float *__restrict__ th, int N, float ih2, float *__restrict__ cof)
+k_cof6f(const __grid_constant__ CofLevels A)
 {
+    int l = 0;
+    while (l + 1 < A.n && blockIdx.x >= A.block[l + 1]) ++l;
+    const int N = A.N[l];
     const size_t n = (size_t)N * N * N;
-    FOR_ROWS(N, i, j)
-    for (int k = threadIdx.x; k < N; k += kRowX) {
-        const Cof<float> a = cofactors(load19<float>(th, N, i, j, k), ih2);
-        const unsigned id = cof_slot(N, i, j, k);
-        cof[id] = a.xx;
-        cof[n + id] = a.yy;
-        cof[2 * n + id] = a.zz;
-        cof[3 * n + id] = a.xy;
-        cof[4 * n + id] = a.yz;
-        cof[5 * n + id] = a.xz;
+    float *cof = A.cof[l];
+    for (unsigned row = (blockIdx.x - A.block[l]) * kRowY + threadIdx.y; row < (unsigned)N * (unsigned)N;
+         row += (A.block[l + 1] - A.block[l]) * kRowY) {
+        const int i = (int)(row / (unsigned)N), j = (int)(row % (unsigned)N);
+        for (int k = threadIdx.x; k < N; k += kRowX) {
+            const Cof<float> a = cofactors(load19<float>(A.th[l], N, i, j, k), A.ih2[l]);
+            const unsigned id = cof_slot(N, i, j, k);
+            cof[id] = a.xx;
+            cof[n + id] = a.yy;
+            cof[2 * n + id] = a.zz;
+            cof[3 * n + id] = a.xy;
+            cof[4 * n + id] = a.yz;
+            cof[5 * n + id] = a.xz;
+        }
     }
+}
+static void add_level(CofLevels &A, int N, double h, const float *th, float *cof)
+{
+    if (A.n == 0) A.block[0] = 0;
+    A.N[A.n] = N;
+    A.ih2[A.n] = (float)(1.0 / (h * h));
+    A.th[A.n] = th;
+    A.cof[A.n] = cof;
+    A.block[A.n + 1] = A.block[A.n] + row_grid(N);
+    ++A.n;
 }
 
 cudaError_t cof6_split(int N, double h, const float *th, float *cof, cudaStream_t s)
 {
+    CofLevels A{};
+    add_level(A, N, h, th, cof);
     note_launch();
-    k_cof6f<<<row_grid(N), row_block(), 0, s>>>(th, N, (float)(1.0 / (h * h)), cof);
+    k_cof6f<<<A.block[A.n], row_block(), 0, s>>>(A);
     return cudaGetLastError();
 }
 
@@ -1403,43 +1542,35 @@ static inline bool lin_fused(int N, const float *e, const float *work)
 // cof: the level's cofactor arrays (read by the two-pass kernels); th: its
 // theta (read by the fused kernel)
 // fshift (nullable): a device scalar subtracted from f on the fly; only the
-// register-blocked kernel takes it (the caller checks lin_fold_ok)
-static cudaError_t lin_sweep(int N, double h, float *e, const float *f, const float *cof,
-                             const float *th, int sweeps, float *work, cudaStream_t s,
-                             const double *fshift = nullptr)
+// register-blocked kernel takes it (the caller checks lin_fold_ok).  zero: e
+// counts as 0 on entry, whatever it holds.  *end (e or w) holds the result.
+static cudaError_t lin_sweep(int N, double h, float *e, float *w, const float *f, const float *cof, const float *th,
+                             int sweeps, cudaStream_t s, const double *fshift, bool zero, float **end)
 {
-    const float ih2 = (float)(1.0 / (h * h));
-    if (reg_sweep_ok(N, e, work, f, th) && reg_sweep_ok(N, work, e, f, th)) {
-        float *a = e, *b = work;
-        for (int it = 0; it < sweeps; ++it) {
-            const cudaError_t err = reg_sweep_launch(true, N, a, b, f, th, nullptr, 0.0, ih2, (float)(h * h / 6.0),
-                                                     0, g_fused_chunk, s, fshift);
-            if (err != cudaSuccess) return err;
-            float *tmp = a;
-            a = b;
-            b = tmp;
-        }
-        if (a != e) return cudaMemcpyAsync(e, a, sizeof(float) * (size_t)N * N * N, cudaMemcpyDeviceToDevice, s);
-        return cudaSuccess;
+    const float ih2 = (float)(1.0 / (h * h)), h2_6 = (float)(h * h / 6.0);
+    const bool reg = reg_sweep_ok(N, e, w, f, th) && reg_sweep_ok(N, w, e, f, th);
+    *end = e;
+    if (zero && (!reg || sweeps == 0)) {
+        const cudaError_t err = cudaMemsetAsync(e, 0, sizeof(float) * (size_t)N * N * N, s);
+        if (err != cudaSuccess) return err;
     }
-    if (lin_fused(N, e, work)) {
-        float *a = e, *b = work;
+    if (reg || lin_fused(N, e, w)) {
         for (int it = 0; it < sweeps; ++it) {
-            const cudaError_t err = fused_sweep_launch<true>(N, a, b, f, th, nullptr, 0.0, ih2,
-                                                                   (float)(h * h / 6.0), 0, s);
+            const cudaError_t err =
+                reg ? reg_sweep_launch(true, N, zero && it == 0 ? nullptr : e, w, f, th, nullptr, 0.0, ih2, h2_6, 0,
+                                       g_fused_chunk, s, fshift)
+                    : fused_sweep_launch<true>(N, e, w, f, th, nullptr, 0.0, ih2, h2_6, 0, s);
             if (err != cudaSuccess) return err;
-            float *tmp = a;
-            a = b;
-            b = tmp;
+            std::swap(e, w);
         }
-        if (a != e) return cudaMemcpyAsync(e, a, sizeof(float) * (size_t)N * N * N, cudaMemcpyDeviceToDevice, s);
+        *end = e;
         return cudaSuccess;
     }
     const dim3 fit = fit_block(N / 2);
     for (int it = 0; it < sweeps; ++it) {
         note_launch(2);
-        k_lin_pass<<<fit_grid(N, fit), fit, 0, s>>>(e, work, f, cof, N, ih2, 0);
-        k_lin_pass<<<fit_grid(N, fit), fit, 0, s>>>(work, e, f, cof, N, ih2, 1);
+        k_lin_pass<<<fit_grid(N, fit), fit, 0, s>>>(e, w, f, cof, N, ih2, 0);
+        k_lin_pass<<<fit_grid(N, fit), fit, 0, s>>>(w, e, f, cof, N, ih2, 1);
     }
     return cudaGetLastError();
 }
@@ -1455,7 +1586,10 @@ cudaError_t linear_sweep(int N, double h, float *e, const float *f, const float 
         const cudaError_t err = cof6_split(N, h, th, cof, s);
         if (err != cudaSuccess) return err;
     }
-    return lin_sweep(N, h, e, f, cof, th, sweeps, work, s);
+    float *end;
+    const cudaError_t err = lin_sweep(N, h, e, work, f, cof, th, sweeps, s, nullptr, false, &end);
+    if (err != cudaSuccess || end == e) return err;
+    return cudaMemcpyAsync(e, end, sizeof(float) * n, cudaMemcpyDeviceToDevice, s);
 }
 
 // fH = R (f - J e), block partial sums for the mean projection, from the
@@ -1466,7 +1600,7 @@ __global__ void __launch_bounds__(kRowThreads, RECON_WIN_CTAS)
 k_lin_restrict_residual(const float *__restrict__ e, const float *__restrict__ f,
                         const float *__restrict__ cof, const float *__restrict__ th, int Nf,
                         float ih2, float *__restrict__ fH, double *__restrict__ partials,
-                        const double *__restrict__ fshift)
+                        const double *__restrict__ fshift, Finish fin)
 {
     __shared__ double sh[32];
     const size_t nf = (size_t)Nf * Nf * Nf;
@@ -1510,8 +1644,10 @@ k_lin_restrict_residual(const float *__restrict__ e, const float *__restrict__ f
         fH[offs(Nc, I, J, K)] = v;
         sacc.add(v);
     }
+    if (!fin.out) return;   // a tail below takes the sum itself
     const double v = block_sum<kRowThreads>(sacc.get(), sh);
     if (ltid() == 0) partials[4 * blockIdx.x + 0] = v;
+    finish_mean<kRowThreads>(partials, fin);
 }
 
 template <typename T, int NT>
@@ -1540,16 +1676,18 @@ namespace {
 template <typename T>
 struct Hier {
     T **t, **g, **told, **aux;
-    T *work;
+    T *const *work;   // per level; null: `scratch` serves all (no kernel leaves an iterate in it)
+    T *scratch;
+    T *w(int l) const { return work ? work[l] : scratch; }
 };
 
 Hier<double> hier64(recon_handle *H)
 {
-    return {H->t64, H->g64, H->told64, H->aux64, H->work64};
+    return {H->t64, H->g64, H->told64, H->aux64, nullptr, H->work64};
 }
 Hier<float> hier32(recon_handle *H)
 {
-    return {H->t32, H->g32, H->told32, H->aux32, H->work32};
+    return {H->t32, H->g32, H->told32, H->aux32, H->work32, nullptr};
 }
 
 inline size_t ncell(int N) { return (size_t)N * N * N; }
@@ -1580,41 +1718,38 @@ cudaError_t vcycle(recon_handle *H, const Hier<T> &Y, int l, const double *cptr,
         }
         return fas_tail<T>(H, l, Y.t[l], Y.g[l], cptr, raw);
     }
-    CK(sweep<T>(N, h, cf.rule, Y.t[l], Y.g[l], cptr, 0.0, cf.nu1, Y.work, s, gshift));
+    T *t = Y.t[l], *w = Y.w(l), *cur, *end;   // the iterate alternates between t and w; it ends in t
+    CK(sweep_from<T>(N, h, cf.rule, t, w, Y.g[l], cptr, 0.0, cf.nu1, s, gshift, &cur));
+    T *const post = sweeps_swap<T>(N, t, w, Y.g[l], nullptr, cf.nu2) ? w : t;
 
     const int Nc = H->Nl[l + 1];
     const size_t nc = ncell(Nc);
-    const unsigned nbr = row_grid(Nc, kMaxRedBlocks);
     note_launch();
-    k_restrict_residual<T><<<nbr, row_block(), 0, s>>>(Y.t[l], Y.g[l], cptr, N, (T)(1.0 / (h * h)),
-                                                    Y.t[l + 1], Y.told[l + 1], Y.g[l + 1],
-                                                    H->partials);
+    k_restrict_residual<T><<<wave_grid(Nc, 2), row_block(), 0, s>>>(cur, Y.g[l], cptr, N, (T)(1.0 / (h * h)),
+                                                    Y.t[l + 1], Y.told[l + 1], Y.g[l + 1], H->partials,
+                                                    Finish{H->ticket, (double)nc,
+                                                           tail_ok<T>(Nc) ? nullptr : H->scal + slot_rmean(l + 1)});
     CK(cudaGetLastError());
+    auto up = [&]() {
+        CK(prolong_to<T>(Nc, Y.t[l + 1], Y.told[l + 1], H->scal + slot_pscale(l + 1), 1.0, cur, post, s));
+        return sweep_from<T>(N, h, cf.rule, post, post == t ? w : t, Y.g[l], cptr, 0.0, cf.nu2, s, nullptr, &end);
+    };
     if (tail_ok<T>(Nc)) {
         CK(vcycle<T>(H, Y, l + 1, H->scal + S_ZERO, nullptr, true));
-        CK(prolong_add<T>(Nc, Y.t[l + 1], Y.told[l + 1], H->scal + slot_pscale(l + 1), 1.0, Y.t[l], s));
-        return sweep<T>(N, h, cf.rule, Y.t[l], Y.g[l], cptr, 0.0, cf.nu2, Y.work, s);
+        return up();
     }
-    note_launch();
-    k_finalize_mean<<<1, kReduceThreads, 0, s>>>(H->partials, nbr, (double)nc,
-                                                 H->scal + slot_rmean(l + 1));
     const double hc = H->hl[l + 1];
     note_launch();
-    k_coarse_rhs<T><<<nbr, row_block(), 0, s>>>(Y.t[l + 1], Y.g[l + 1], Y.aux[l + 1],
+    k_coarse_rhs<T><<<wave_grid(Nc, 4), row_block(), 0, s>>>(Y.t[l + 1], Y.g[l + 1], Y.aux[l + 1],
                                              H->scal + slot_rmean(l + 1), Nc,
-                                             (T)(1.0 / (hc * hc)), cf.scale_floor, H->partials);
-    note_launch();
-    k_finalize_scale<<<1, kReduceThreads, 0, s>>>(H->partials, nbr, cf.scale_floor,
-                                                  H->scal + slot_scale(l + 1),
-                                                  H->scal + slot_pscale(l + 1));
+                                             (T)(1.0 / (hc * hc)), cf.scale_floor, H->partials,
+                                             Finish{H->ticket, (double)nc, H->scal + slot_scale(l + 1)});
     note_launch();
     k_form_rhs<T><<<stride_blocks(nc), kThreads, 0, s>>>(Y.g[l + 1], Y.aux[l + 1], nc,
                                                       H->scal + slot_scale(l + 1));
     CK(cudaGetLastError());
     CK(vcycle<T>(H, Y, l + 1, H->scal + S_ZERO));
-    CK(prolong_add<T>(Nc, Y.t[l + 1], Y.told[l + 1], H->scal + slot_pscale(l + 1), 1.0,
-                      Y.t[l], s));
-    return sweep<T>(N, h, cf.rule, Y.t[l], Y.g[l], cptr, 0.0, cf.nu2, Y.work, s);
+    return up();
 }
 
 // residual norms of level l, then c -= mean r, rel, and theta -= mean theta
@@ -1627,10 +1762,7 @@ cudaError_t compat_gauge(recon_handle *H, const Hier<T> &Y, int l, bool apply = 
     const int N = H->Nl[l];
     const size_t n = ncell(N);
     const double h = H->hl[l];
-    const unsigned nbr = launch_residual_norms<T>(Y.t[l], Y.g[l], H->scal + S_C, N, (T)(1.0 / (h * h)),
-                                                  H->partials, nullptr, nullptr, s);
-    note_launch();
-    k_finalize_cycle<<<1, kReduceThreads, 0, s>>>(H->partials, nbr, (double)n, H->scal);
+    CK(residual_norms<T>(H, Y.t[l], Y.g[l], N, (T)(1.0 / (h * h)), nullptr, nullptr));
     if (apply) {
         note_launch();
         k_gauge<T><<<stride_blocks(n), kThreads, 0, s>>>(Y.t[l], n, H->scal);
@@ -1645,7 +1777,7 @@ cudaError_t fmg_start(recon_handle *H, const Hier<T> &Y)
 {
     cudaStream_t s = H->stream;
     const int lc = H->nlev - 1;
-    for (int l = 1; l <= lc; ++l) CK(restrict_plain<T>(H->Nl[l - 1], Y.g[l - 1], Y.g[l], s));
+    CK(restrict_levels<T>(H->Nl, H->nlev, Y.g, s));
     CK(cudaMemsetAsync(Y.t[lc], 0, sizeof(T) * ncell(H->Nl[lc]), s));
     CK(cudaMemsetAsync(H->scal + S_C, 0, sizeof(double), s));
     CK(vcycle<T>(H, Y, lc, H->scal + S_C));
@@ -1688,11 +1820,8 @@ void hist_push(recon_stats *st, double v)
 recon_status check_domain(recon_handle *H, const double *b)
 {
     const size_t n = ncell(H->N);
-    const unsigned nbr = red_blocks(n);
     note_launch();
-    k_b_stats<<<nbr, kThreads, 0, H->stream>>>(b, n, H->partials);
-    note_launch();
-    k_finalize_b<<<1, kReduceThreads, 0, H->stream>>>(H->partials, nbr, H->scal);
+    k_b_stats<<<red_blocks(n), kThreads, 0, H->stream>>>(b, n, H->partials, Finish{H->ticket, (double)n, H->scal});
     cudaError_t e = cudaGetLastError();
     if (e == cudaSuccess) e = read_scalars(H);
     if (e != cudaSuccess) return fail_cuda(H, e, "domain check");
@@ -1776,15 +1905,15 @@ static bool lin_fold_ok(recon_handle *H, int l)
 {
     const int N = H->Nl[l];
     return l < H->nlev - 1 && !tail_ok<float>(N) &&
-           reg_sweep_ok(N, H->e32[l], H->work32, H->f32[l], H->t32[l]) &&
-           reg_sweep_ok(N, H->work32, H->e32[l], H->f32[l], H->t32[l]);
+           reg_sweep_ok(N, H->e32[l], H->work32[l], H->f32[l], H->t32[l]) &&
+           reg_sweep_ok(N, H->work32[l], H->e32[l], H->f32[l], H->t32[l]);
 }
 
 // fshift (nullable, level l only): a device scalar subtracted from f on the
 // fly by the register-blocked sweep and the restriction (lin_fold_ok).
-// raw: f still carries its mean and e is not yet zeroed (only where a tail
-// starts, which does both).
-cudaError_t lin_vcycle(recon_handle *H, int l, const double *fshift = nullptr, bool raw = false)
+// raw: f still carries its mean (only where a tail starts, which removes it).
+// zero: e counts as 0 on entry, whatever it holds.
+cudaError_t lin_vcycle(recon_handle *H, int l, const double *fshift, bool raw, bool zero)
 {
     cudaStream_t s = H->stream;
     const recon_config &cf = H->cfg;
@@ -1792,37 +1921,41 @@ cudaError_t lin_vcycle(recon_handle *H, int l, const double *fshift = nullptr, b
     const int N = H->Nl[l];
     const double h = H->hl[l];
     const float ih2 = (float)(1.0 / (h * h));
-    if (tail_ok<float>(N)) return lin_tail(H, l, H->e32[l], H->f32[l], H->cof32, raw, raw);
-    CK(lin_sweep(N, h, H->e32[l], H->f32[l], H->cof32[l], H->t32[l], cf.nu1, H->work32, s, fshift));
+    if (tail_ok<float>(N)) return lin_tail(H, l, H->e32[l], H->f32[l], H->cof32, raw, zero);
+    float *e = H->e32[l], *w = H->work32[l], *const f = H->f32[l], *const th = H->t32[l], *cur, *end;
+    // the iterate alternates between e and w and ends in e; a first sweep from
+    // e = 0 reads neither, so it starts where the prolongation is in place
+    float *const post = sweeps_swap<float>(N, e, w, f, th, cf.nu2) ? w : e;
+    const bool flip = zero && (sweeps_swap<float>(N, e, w, f, th, cf.nu1) ? post == e : post == w);
+    CK(lin_sweep(N, h, flip ? w : e, flip ? e : w, f, H->cof32[l], th, cf.nu1, s, fshift, zero, &cur));
     const int Nc = H->Nl[l + 1];
     const size_t nc = ncell(Nc);
-    const unsigned nbr = row_grid(Nc, kMaxRedBlocks);
+    const unsigned nbr = wave_grid(Nc, 2);
+    const Finish fin = {H->ticket, (double)nc, tail_ok<float>(Nc) ? nullptr : H->scal + slot_rmean(l + 1)};
     note_launch();
     if (H->cof32[l])
-        k_lin_restrict_residual<false><<<nbr, row_block(), 0, s>>>(H->e32[l], H->f32[l], H->cof32[l], nullptr,
-                                                                    N, ih2, H->f32[l + 1], H->partials, fshift);
+        k_lin_restrict_residual<false><<<nbr, row_block(), 0, s>>>(cur, H->f32[l], H->cof32[l], nullptr,
+                                                                    N, ih2, H->f32[l + 1], H->partials, fshift, fin);
     else
-        k_lin_restrict_residual<true><<<nbr, row_block(), 0, s>>>(H->e32[l], H->f32[l], nullptr, H->t32[l],
-                                                                   N, ih2, H->f32[l + 1], H->partials, fshift);
+        k_lin_restrict_residual<true><<<nbr, row_block(), 0, s>>>(cur, H->f32[l], nullptr, H->t32[l],
+                                                                   N, ih2, H->f32[l + 1], H->partials, fshift, fin);
     CK(cudaGetLastError());
+    auto up = [&]() {
+        CK(prolong_to<float>(Nc, H->e32[l + 1], nullptr, nullptr, 1.0, cur, post, s));
+        return lin_sweep(N, h, post, post == e ? w : e, f, H->cof32[l], th, cf.nu2, s, fshift, false, &end);
+    };
     if (tail_ok<float>(Nc)) {
-        CK(lin_vcycle(H, l + 1, nullptr, true));
-        CK(prolong_add<float>(Nc, H->e32[l + 1], (const float *)nullptr, nullptr, 1.0, H->e32[l], s));
-        return lin_sweep(N, h, H->e32[l], H->f32[l], H->cof32[l], H->t32[l], cf.nu2, H->work32, s, fshift);
+        CK(lin_vcycle(H, l + 1, nullptr, true, true));
+        return up();
     }
-    note_launch();
-    k_finalize_mean<<<1, kReduceThreads, 0, s>>>(H->partials, nbr, (double)nc,
-                                                 H->scal + slot_rmean(l + 1));
     // f - mean f on the coarse level: folded into its kernels where they can
     const bool fold = lin_fold_ok(H, l + 1);
     if (!fold) {
         note_launch();
         k_sub_scalar<<<stride_blocks(nc), kThreads, 0, s>>>(H->f32[l + 1], nc, H->scal + slot_rmean(l + 1));
     }
-    CK(cudaMemsetAsync(H->e32[l + 1], 0, sizeof(float) * nc, s));
-    CK(lin_vcycle(H, l + 1, fold ? H->scal + slot_rmean(l + 1) : nullptr));
-    CK(prolong_add<float>(Nc, H->e32[l + 1], (const float *)nullptr, nullptr, 1.0, H->e32[l], s));
-    return lin_sweep(N, h, H->e32[l], H->f32[l], H->cof32[l], H->t32[l], cf.nu2, H->work32, s, fshift);
+    CK(lin_vcycle(H, l + 1, fold ? H->scal + slot_rmean(l + 1) : nullptr, false, true));
+    return up();
 }
 
 
@@ -1890,13 +2023,15 @@ cudaError_t mixed_residual(recon_handle *H, const double *b, const double *phi)
 {
     cudaStream_t s = H->stream;
     const size_t n = ncell(H->N);
-    unsigned nbr = row_grid(H->N, kMaxRedBlocks);
+    // (2048 blocks and a second launch for the scalars: one wave of 608 blocks
+    // that ends in last_block took 2.42 ms at 512^3, many short ones 2.03)
+    const unsigned nbr = row_grid(H->N, kMaxRedBlocks);
     const double ih2 = 1.0 / (H->h * H->h);
     if (H->cfg.mixed_df_residual) {
         const df ih2df = df_from_double(ih2);
         int ex;
         const bool pow2 = ih2df.lo == 0.0f && std::frexp(ih2, &ex) == 0.5;
-        note_launch();
+        note_launch(2);
         if (pow2)
             k_residual_df<true><<<nbr, row_block(), 0, s>>>(H->t32[0], H->lo32, H->g32[0], H->blo32,
                                                             H->scal + S_C, H->N, ih2df.hi, ih2df.lo,
@@ -1905,12 +2040,10 @@ cudaError_t mixed_residual(recon_handle *H, const double *b, const double *phi)
             k_residual_df<false><<<nbr, row_block(), 0, s>>>(H->t32[0], H->lo32, H->g32[0], H->blo32,
                                                              H->scal + S_C, H->N, ih2df.hi, ih2df.lo,
                                                              H->f32[0], H->partials);
+        k_finish_cycle<<<1, kRowThreads, 0, s>>>(H->partials, (int)nbr, (double)n, H->scal);
     } else {
-        nbr = launch_residual_norms<double>(phi, b, H->scal + S_C, H->N, ih2, H->partials, H->f32[0],
-                                            H->t32[0], s);
+        CK(residual_norms<double>(H, phi, b, H->N, ih2, H->f32[0], H->t32[0]));
     }
-    note_launch();
-    k_finalize_cycle<<<1, kReduceThreads, 0, s>>>(H->partials, nbr, (double)n, H->scal);
     return cudaGetLastError();
 }
 
@@ -1926,14 +2059,14 @@ cudaError_t mixed_correct(recon_handle *H, double *phi)
         note_launch();
         k_sub_scalar<<<stride_blocks(n), kThreads, 0, s>>>(H->f32[0], n, H->scal + S_MEAN_R);
     }
-    for (int l = 1; l < H->nlev; ++l) CK(restrict_plain<float>(H->Nl[l - 1], H->t32[l - 1], H->t32[l], s));
-    for (int l = 0; l < H->nlev; ++l) {
-        if (H->Nl[l] >= kFusedMinN) continue;   // formed from theta32 in the kernels
-        CK(cof6_split(H->Nl[l], H->hl[l], H->t32[l], H->cof32[l], s));
-    }
-    CK(cudaMemsetAsync(H->e32[0], 0, sizeof(float) * n, s));
+    CK(restrict_levels<float>(H->Nl, H->nlev, H->t32, s));
+    CofLevels A{};   // (larger grids form them from theta32 in their kernels)
+    for (int l = 0; l < H->nlev; ++l)
+        if (H->Nl[l] < kFusedMinN) add_level(A, H->Nl[l], H->hl[l], H->t32[l], H->cof32[l]);
+    note_launch();
+    k_cof6f<<<A.block[A.n], row_block(), 0, s>>>(A);
     for (int v = 0; v < H->cfg.mixed_linear_vcycles; ++v)
-        CK(lin_vcycle(H, 0, fold ? H->scal + S_MEAN_R : nullptr));
+        CK(lin_vcycle(H, 0, fold ? H->scal + S_MEAN_R : nullptr, false, v == 0));
     note_launch();
     if (H->cfg.mixed_df_residual)
         k_update_df<<<blocks_for(n), kThreads, 0, s>>>(H->t32[0], H->lo32, H->e32[0], n);
@@ -1948,10 +2081,9 @@ cudaError_t mixed_finish(recon_handle *H, double *phi, bool converged)
     cudaStream_t s = H->stream;
     const size_t n = ncell(H->N);
     if (H->cfg.mixed_df_residual) {
-        const unsigned nb2 = red_blocks(n);
-        note_launch(3);
-        k_df_sum<<<nb2, kThreads, 0, s>>>(H->t32[0], H->lo32, n, H->partials);
-        k_finalize_mean<<<1, kReduceThreads, 0, s>>>(H->partials, nb2, (double)n, H->scal + S_MEAN_T);
+        note_launch(2);
+        k_df_sum<<<red_blocks(n), kThreads, 0, s>>>(H->t32[0], H->lo32, n, H->partials,
+                                                    Finish{H->ticket, (double)n, H->scal + S_MEAN_T});
         k_df_to_double_gauged<<<stride_blocks(n), kThreads, 0, s>>>(H->t32[0], H->lo32, phi, n,
                                                                    H->scal + S_MEAN_T);
     } else if (converged) {

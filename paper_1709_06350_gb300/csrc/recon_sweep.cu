@@ -44,41 +44,44 @@ namespace recon {
 namespace {
 
 constexpr int kBK = 64;                          // tile columns (k)
-constexpr int kBJ = 16;                          // tile rows (j)
-constexpr int kCW = kBJ / 2;                     // warps
-constexpr int kBT = 32 * kCW;                    // threads
 constexpr int kHOH = (kBK + 4) / 2;              // 34 positions of one k parity per OLD row
 constexpr int kHOW = 2 * kHOH;                   // 68 staged positions per OLD row
 constexpr int kHOR = kHOW + 1;                   // OLD row stride: odd, so that the ring columns'
                                                  // cells (rows 2 apart) hit distinct banks
-constexpr int kHOJ = kBJ + 4;                    // 20 OLD rows
-constexpr int kHOP = kHOJ * kHOR;                // OLD plane stride (floats)
-constexpr int kHOS = kHOJ * kHOW;                // 1360 staged positions per OLD plane
 constexpr int kHRH = kBK / 2 + 1;                // 33 red cells per RED row
-constexpr int kHRJ = kBJ + 2;                    // 18 RED rows
-constexpr int kHRP = kHRJ * kHRH;                // 594 per RED plane
-constexpr int kGT = kBJ * kBK;                   // right-side values of the tile per plane
-constexpr int kGP = kGT + 2 * kBK + 2 * kBJ;     // ... and of the ring (rows -1, kBJ; columns -1, kBK)
 constexpr int kSlots = 6;                        // planes s-1 .. s+2 in use, s+3 and s+4 in flight
-constexpr int kStage = (kHOS + kBT - 1) / kBT;   // OLD positions staged per thread per plane
 constexpr unsigned kNoStage = 0xFFFu;            // packed staging position: none
-static_assert(kBK / 2 == 32 && kGT / 4 == kBT && kBK / 4 == 16 && kBJ == 16,
-              "lane m owns columns 2m, 2m+1; one 16-byte copy of the tile's right side per thread; "
-              "warp 7 copies the ring's right side in two instructions");
-static_assert((kStage - 1) * kBT <= kHOS, "only the last staging round can run past the plane");
-static_assert(kHOP < (int)kNoStage && kMaxN * kMaxN <= (1 << 20), "staging offsets are packed into 12 + 20 bits");
 
-// A slot holds one OLD plane (LIN: the e plane, then the theta plane)
-// followed by the same plane's right side (floats).
-template <bool LIN>
-__host__ __device__ constexpr int slot_floats() { return (LIN ? 2 : 1) * kHOP + kGP; }
-template <bool LIN>
-__host__ __device__ constexpr int g_off() { return (LIN ? 2 : 1) * kHOP; }
-template <bool LIN>
-__host__ __device__ constexpr size_t reg_smem_bytes() { return 4u * ((size_t)kSlots * slot_floats<LIN>() + 2u * kHRP); }
-static_assert(slot_floats<false>() % 4 == 0 && slot_floats<true>() % 4 == 0 && g_off<false>() % 4 == 0 &&
-                  g_off<true>() % 4 == 0,
-              "16-byte copies of the right side need 16-byte aligned slots");
+// What a sweep relaxes: the cell cubic, J e = f, or J e = f from e = 0
+enum Mode { FAS, LIN, LIN0 };
+
+// Tile and shared-memory layout of a CTA
+template <Mode M>
+struct Tile {
+    static constexpr int kBJ = 16;                          // tile rows (j)
+    static constexpr int kCW = kBJ / 2;                     // warps
+    static constexpr int kBT = 32 * kCW;                    // threads
+    static constexpr int kHOJ = kBJ + 4;                    // OLD rows
+    static constexpr int kHOP = kHOJ * kHOR;                // OLD plane stride (floats)
+    static constexpr int kHOS = kHOJ * kHOW;                // staged positions per OLD plane
+    static constexpr int kHRJ = kBJ + 2;                    // RED rows
+    static constexpr int kHRP = kHRJ * kHRH;                // per RED plane
+    static constexpr int kGT = kBJ * kBK;                   // right-side values of the tile per plane
+    static constexpr int kGP = kGT + 2 * kBK + 2 * kBJ;     // ... and of the ring (rows -1, kBJ; columns -1, kBK)
+    static constexpr int kStage = (kHOS + kBT - 1) / kBT;   // OLD positions staged per thread per plane
+    static_assert(kBK / 2 == 32 && kGT / 4 == kBT && kBK / 4 == 16 && kBJ <= 16,
+                  "lane m owns columns 2m, 2m+1; one 16-byte copy of the tile's right side per thread; the last "
+                  "warp copies the ring's right side in two instructions");
+    static_assert((kStage - 1) * kBT <= kHOS, "only the last staging round can run past the plane");
+    static_assert(kHOP < (int)kNoStage && kMaxN * kMaxN <= (1 << 20), "staging offsets are packed into 12 + 20 bits");
+    // A slot holds the OLD planes (FAS: theta; LIN: e, then theta; LIN0: theta)
+    // followed by the same plane's right side (floats).
+    static constexpr int kPlanes = M == LIN ? 2 : 1;
+    static constexpr int kTheta = M == LIN ? kHOP : 0;      // offset of theta's plane in a slot (LIN, LIN0)
+    static constexpr int kG = (kPlanes * kHOP + 3) / 4 * 4; // ... of the right side (16-byte copies)
+    static constexpr int kSlot = kG + (kGP + 3) / 4 * 4;
+    static constexpr size_t kSmem = 4u * ((size_t)kSlots * kSlot + 2u * kHRP);
+};
 
 // the sweep's dynamic shared memory, addressed by float index
 extern __shared__ __align__(16) float rsm[];
@@ -197,12 +200,15 @@ __device__ __forceinline__ Nb19<float> gather_at(int pm, int pc, int pp, int S, 
     return v;
 }
 
-// OLD-plane offset of the tile cell (jl, kl), jl in [-2, kBJ + 1], kl in [-2, kBK + 1]
+// OLD-plane offset of the tile cell (jl, kl), jl in [-2, rows + 1], kl in [-2, kBK + 1]
 __device__ __forceinline__ int opos(int jl, int kl) { return (jl + 2) * kHOR + (kl & 1) * kHOH + ((kl + 2) >> 1); }
 
 // ---- the sweep ------------------------------------------------------------
-template <bool LIN>
+template <Mode M>
 struct RegSweep {
+    using Tl = Tile<M>;
+    static constexpr int kBJ = Tl::kBJ, kCW = Tl::kCW, kHOP = Tl::kHOP, kHRP = Tl::kHRP, kGT = Tl::kGT;
+    static constexpr int kStage = Tl::kStage, kTheta = Tl::kTheta;
     const float *src, *th, *g;
     float *dst;
     int N;
@@ -234,11 +240,11 @@ struct RegSweep {
             for (int x = 0; x < kStage; ++x)
                 if (x < kStage - 1 || (stg[x] >> 20) != kNoStage) {
                     const unsigned so4 = sb + 4u * (stg[x] >> 20), go = pb + (stg[x] & 0xFFFFFu);
-                    cpa4(so4, src + go);
-                    if constexpr (LIN) cpa4(so4 + 4u * kHOP, th + go);
+                    cpa4(so4, (M == LIN0 ? th : src) + go);
+                    if constexpr (M == LIN) cpa4(so4 + 4u * kTheta, th + go);
                 }
             if (q <= i1 && q >= i0 - 1) {
-                const unsigned gs = sb + 4u * (unsigned)g_off<LIN>();
+                const unsigned gs = sb + 4u * (unsigned)Tl::kG;
                 const int tid = 32 * w + lane, row = tid >> 4, col = (tid & 15) * 4;
                 cpa16(gs + 4u * (unsigned)(row * kBK + col),
                       g + pb + (unsigned)(j0 + row) * (unsigned)N + (unsigned)(k0 + col));
@@ -248,8 +254,9 @@ struct RegSweep {
                     const unsigned jr = (unsigned)wrapn(hi ? j0 + kBJ : j0 - 1, N);
                     cpa16(gs + 4u * (unsigned)(kGT + hi * kBK + c4), g + pb + jr * (unsigned)N + (unsigned)(k0 + c4));
                     const unsigned kc = (unsigned)wrapn(hi ? k0 + kBK : k0 - 1, N);
-                    cpa4(gs + 4u * (unsigned)(kGT + 2 * kBK + hi * kBJ + (lane & 15)),
-                         g + pb + (unsigned)(j0 + (lane & 15)) * (unsigned)N + kc);
+                    if ((lane & 15) < kBJ)
+                        cpa4(gs + 4u * (unsigned)(kGT + 2 * kBK + hi * kBJ + (lane & 15)),
+                             g + pb + (unsigned)(j0 + (lane & 15)) * (unsigned)N + kc);
                 }
             }
         }
@@ -260,15 +267,17 @@ struct RegSweep {
     __device__ __forceinline__ void load_own(int so)
     {
         const int b = so + tb;
-        v[Q][0] = rsm[b + 1];
-        v[Q][1] = rsm[b + kHOH + 1];
-        v[Q][2] = rsm[b + kHOR + 1];
-        v[Q][3] = rsm[b + kHOR + kHOH + 1];
-        if constexpr (LIN) {
-            t[Q][0] = rsm[b + kHOP + 1];
-            t[Q][1] = rsm[b + kHOP + kHOH + 1];
-            t[Q][2] = rsm[b + kHOP + kHOR + 1];
-            t[Q][3] = rsm[b + kHOP + kHOR + kHOH + 1];
+        if constexpr (M != LIN0) {
+            v[Q][0] = rsm[b + 1];
+            v[Q][1] = rsm[b + kHOH + 1];
+            v[Q][2] = rsm[b + kHOR + 1];
+            v[Q][3] = rsm[b + kHOR + kHOH + 1];
+        }
+        if constexpr (M != FAS) {
+            t[Q][0] = rsm[b + kTheta + 1];
+            t[Q][1] = rsm[b + kTheta + kHOH + 1];
+            t[Q][2] = rsm[b + kTheta + kHOR + 1];
+            t[Q][3] = rsm[b + kTheta + kHOR + kHOH + 1];
         }
     }
 
@@ -282,22 +291,28 @@ struct RegSweep {
     __device__ __forceinline__ void red_own(int som, int soc, int sop)
     {
         constexpr int B0 = P, B1 = 1 - P;
-        const int gp = soc + g_off<LIN>() + 2 * w * kBK + 2 * lane;
+        const int gp = soc + Tl::kG + 2 * w * kBK + 2 * lane;
         const float2 g0 = *reinterpret_cast<const float2 *>(&rsm[gp]);
         const float2 g1 = *reinterpret_cast<const float2 *>(&rsm[gp + kBK]);
         const float2 rhs = make_float2(B0 ? g0.y : g0.x, B1 ? g1.y : g1.x);
         gb[P][0] = B0 ? g0.x : g0.y;
         gb[P][1] = B1 ? g1.x : g1.y;
         const int pm = som + tb, pc = soc + tb, pp = sop + tb;
-        const Nb19<float> n0 = old19<QM, Q0, QP, 0, B0>(v, pm, pc, pp);
-        const Nb19<float> n1 = old19<QM, Q0, QP, 1, B1>(v, pm, pc, pp);
         float2 out;
-        if constexpr (LIN) {
-            const Nb19<float> t0 = old19<QM, Q0, QP, 0, B0>(t, pm + kHOP, pc + kHOP, pp + kHOP);
-            const Nb19<float> t1 = old19<QM, Q0, QP, 1, B1>(t, pm + kHOP, pc + kHOP, pp + kHOP);
-            out = lin_update2(pack19(t0, t1), pack19(n0, n1), add2(rhs, f2(c)), ih2, 6.0f * h2_6);
-        } else {
+        if constexpr (M == FAS) {
+            const Nb19<float> n0 = old19<QM, Q0, QP, 0, B0>(v, pm, pc, pp);
+            const Nb19<float> n1 = old19<QM, Q0, QP, 1, B1>(v, pm, pc, pp);
             out = fas_update2_det(pack19(n0, n1), add2(rhs, f2(c)), ih2, 3.0f * h2_6, h2_6, rule);
+        } else {
+            const Nb19<float> t0 = old19<QM, Q0, QP, 0, B0>(t, pm + kTheta, pc + kTheta, pp + kTheta);
+            const Nb19<float> t1 = old19<QM, Q0, QP, 1, B1>(t, pm + kTheta, pc + kTheta, pp + kTheta);
+            if constexpr (M == LIN) {
+                const Nb19<float> n0 = old19<QM, Q0, QP, 0, B0>(v, pm, pc, pp);
+                const Nb19<float> n1 = old19<QM, Q0, QP, 1, B1>(v, pm, pc, pp);
+                out = lin_update2(pack19(t0, t1), pack19(n0, n1), add2(rhs, f2(c)), ih2, 6.0f * h2_6);
+            } else {
+                out = lin_update2_zero(pack19(t0, t1), add2(rhs, f2(c)), ih2, 6.0f * h2_6);
+            }
         }
         r[Q0][B0] = out.x;
         r[Q0][2 + B1] = out.y;
@@ -314,24 +329,33 @@ struct RegSweep {
         constexpr int B0 = 1 - P, B1 = P;
         const int pm = som + tb, pc = soc + tb, pp = sop + tb;
         const int rp = P * kHRP + rb;
-        const Nb19<float> n0 = old19<QM, Q0, QP, 0, B0>(v, pm, pc, pp);
-        const Nb19<float> n1 = old19<QM, Q0, QP, 1, B1>(v, pm, pc, pp);
         const float2 rhs = make_float2(gb[P][0], gb[P][1]);
-        Nb19<float> a0 = n0, a1 = n1;
+        Nb19<float> a0, a1;
+        if constexpr (M != LIN0) {
+            a0 = old19<QM, Q0, QP, 0, B0>(v, pm, pc, pp);
+            a1 = old19<QM, Q0, QP, 1, B1>(v, pm, pc, pp);
+        }
         red_faces<QM, Q0, QP, 0, B0>(a0, r, rp);
         red_faces<QM, Q0, QP, 1, B1>(a1, r, rp);
         float2 out;
-        if constexpr (LIN) {
-            const Nb19<float> t0 = old19<QM, Q0, QP, 0, B0>(t, pm + kHOP, pc + kHOP, pp + kHOP);
-            const Nb19<float> t1 = old19<QM, Q0, QP, 1, B1>(t, pm + kHOP, pc + kHOP, pp + kHOP);
-            out = lin_update2(pack19(t0, t1), pack19(a0, a1), add2(rhs, f2(c)), ih2, 6.0f * h2_6);
-        } else {
+        if constexpr (M == FAS) {
             out = fas_update2_det(pack19(a0, a1), add2(rhs, f2(c)), ih2, 3.0f * h2_6, h2_6, rule);
+        } else {
+            const Nb19<float> t0 = old19<QM, Q0, QP, 0, B0>(t, pm + kTheta, pc + kTheta, pp + kTheta);
+            const Nb19<float> t1 = old19<QM, Q0, QP, 1, B1>(t, pm + kTheta, pc + kTheta, pp + kTheta);
+            if constexpr (M == LIN) {
+                out = lin_update2(pack19(t0, t1), pack19(a0, a1), add2(rhs, f2(c)), ih2, 6.0f * h2_6);
+            } else {
+                const float2 sx = add2(make_float2(a0.xp, a1.xp), make_float2(a0.xm, a1.xm));
+                const float2 sy = add2(make_float2(a0.yp, a1.yp), make_float2(a0.ym, a1.ym));
+                const float2 sz = add2(make_float2(a0.zp, a1.zp), make_float2(a0.zm, a1.zm));
+                out = lin_update2_faces(pack19(t0, t1), sx, sy, sz, add2(rhs, f2(c)), ih2, 6.0f * h2_6);
+            }
         }
         const unsigned base = (unsigned)s * NN + gown;
         float2 row0 = B0 ? make_float2(r[Q0][0], out.x) : make_float2(out.x, r[Q0][1]);
         float2 row1 = B1 ? make_float2(r[Q0][2], out.y) : make_float2(out.y, r[Q0][3]);
-        if constexpr (!LIN) {
+        if constexpr (M == FAS) {
             row0 = sub2(row0, f2(gsh));
             row1 = sub2(row1, f2(gsh));
         }
@@ -365,20 +389,26 @@ struct RegSweep {
         }
         const int Sa = opos(ja, ka), Oa = opos(ja, ka - 1);
         const int Sb = opos(jb, kb), Ob = opos(jb, kb - 1);
-        const Nb19<float> na = gather_at(som, soc, sop, Sa, Oa);
-        const Nb19<float> nb = gather_at(som, soc, sop, Sb, Ob);
-        const int gs = soc + g_off<LIN>();
+        const int gs = soc + Tl::kG;
         const float2 rhs = make_float2(rsm[gs + ga], rsm[gs + gbi]);
         float2 out;
-        if constexpr (LIN) {
-            const Nb19<float> ta = gather_at(som + kHOP, soc + kHOP, sop + kHOP, Sa, Oa);
-            const Nb19<float> tb_ = gather_at(som + kHOP, soc + kHOP, sop + kHOP, Sb, Ob);
-            out = lin_update2(pack19(ta, tb_), pack19(na, nb), add2(rhs, f2(c)), ih2, 6.0f * h2_6);
-        } else {
+        if constexpr (M == FAS) {
+            const Nb19<float> na = gather_at(som, soc, sop, Sa, Oa);
+            const Nb19<float> nb = gather_at(som, soc, sop, Sb, Ob);
             out = fas_update2_det(pack19(na, nb), add2(rhs, f2(c)), ih2, 3.0f * h2_6, h2_6, rule);
+        } else {
+            const Nb19<float> ta = gather_at(som + kTheta, soc + kTheta, sop + kTheta, Sa, Oa);
+            const Nb19<float> tb_ = gather_at(som + kTheta, soc + kTheta, sop + kTheta, Sb, Ob);
+            if constexpr (M == LIN) {
+                const Nb19<float> na = gather_at(som, soc, sop, Sa, Oa);
+                const Nb19<float> nb = gather_at(som, soc, sop, Sb, Ob);
+                out = lin_update2(pack19(ta, tb_), pack19(na, nb), add2(rhs, f2(c)), ih2, 6.0f * h2_6);
+            } else {
+                out = lin_update2_zero(pack19(ta, tb_), add2(rhs, f2(c)), ih2, 6.0f * h2_6);
+            }
         }
         if (PAIR == 0 || lane < kBJ / 2) {
-            const int rbase = kSlots * slot_floats<LIN>() + P * kHRP;
+            const int rbase = kSlots * Tl::kSlot + P * kHRP;
             rsm[rbase + (ja + 1) * kHRH + ((ka + 1) >> 1)] = out.x;
             rsm[rbase + (jb + 1) * kHRH + ((kb + 1) >> 1)] = out.y;
         }
@@ -411,7 +441,7 @@ struct RegSweep {
         // prologue: OLD planes i0-2 .. i0+2 (and right sides i0-1 .. i0+2) in
         // slots 0..4, plane i0+3 in flight into slot 5
 #pragma unroll
-        for (int d = 0; d < kSlots; ++d) sl[d] = d * slot_floats<LIN>();
+        for (int d = 0; d < kSlots; ++d) sl[d] = d * Tl::kSlot;
 #pragma unroll
         for (int d = 0; d < kSlots; ++d) issue(i0 - 2 + d, sl[d]);
         cpa_wait<1>();
@@ -441,22 +471,24 @@ struct RegSweep {
     }
 };
 
-// CTAs per SM: FAS 2 (four warps per scheduler, 128 registers); LIN 1 (its
-// e and theta neighbourhoods need ~180 registers, and spilling cost more than
-// the lower occupancy: 512^3 sweep 1.13 ms at two CTAs, 0.88 ms at one)
-#ifndef RECON_REG_CTAS_FAS
-#define RECON_REG_CTAS_FAS 2
-#endif
-#ifndef RECON_REG_CTAS_LIN
-#define RECON_REG_CTAS_LIN 1
-#endif
-template <bool LIN>
-__global__ void __launch_bounds__(kBT, LIN ? RECON_REG_CTAS_LIN : RECON_REG_CTAS_FAS)
+// CTAs per SM: FAS and LIN0 2 (four warps per scheduler, 128 registers); LIN 1
+// (its e and theta neighbourhoods need ~180 registers, and spilling cost more
+// than the lower occupancy: 512^3 sweep 1.13 ms at two CTAs, 0.87 ms at one;
+// half the rows, for two or three CTAs of four warps at 168 registers, 0.95 and
+// 1.10 ms, their rings' loads; 12 rows with two warps for the ring alone, 146
+// registers, 1.22 ms at one CTA and 1.07 ms at two).  From e = 0 (LIN0) the
+// centre, the edges and the off-diagonal cofactors drop out:
+// 512^3 0.51 ms against 0.87 ms for a sweep of a zeroed e, which cost another
+// 0.08 ms to zero; 256^3 79 against 132 us.
+template <Mode M>
+__global__ void __launch_bounds__(Tile<M>::kBT, M == LIN ? 1 : 2)
 k_sweep_reg(const float *__restrict__ src, float *__restrict__ dst, const float *__restrict__ g,
             const float *__restrict__ th, const double *__restrict__ cptr, double cval, int N, int CI,
             float ih2, float h2_6, int rule, const double *__restrict__ gshift)
 {
-    RegSweep<LIN> S;
+    using Tl = Tile<M>;
+    constexpr int kHOS = Tl::kHOS, kBJ = Tl::kBJ;
+    RegSweep<M> S;
     S.src = src;
     S.th = th;
     S.g = g;
@@ -471,8 +503,8 @@ k_sweep_reg(const float *__restrict__ src, float *__restrict__ dst, const float 
     S.h2_6 = h2_6;
     // FAS: the compatibility scalar c added to the right side; LIN: minus the
     // shift subtracted from f (its mean, folded in: f + (-m) rounds as f - m)
-    S.c = LIN ? (gshift ? -(float)*gshift : 0.0f) : (float)(cptr ? *cptr : cval);
-    S.gsh = (!LIN && gshift) ? (float)*gshift : 0.0f;
+    S.c = M != FAS ? (gshift ? -(float)*gshift : 0.0f) : (float)(cptr ? *cptr : cval);
+    S.gsh = (M == FAS && gshift) ? (float)*gshift : 0.0f;
     S.rule = rule;
     const int tid = threadIdx.x;
     // the warp index through a shuffle from lane 0: the compiler sees it as
@@ -480,14 +512,14 @@ k_sweep_reg(const float *__restrict__ src, float *__restrict__ dst, const float 
     S.w = __shfl_sync(0xffffffffu, tid >> 5, 0);
     S.lane = tid & 31;
     S.hrow = S.w == 0;
-    S.hcol = S.w == kCW - 1;
+    S.hcol = S.w == Tl::kCW - 1;
     S.tb = (2 * S.w + 2) * kHOR + S.lane;
-    S.rb = (2 * S.w + 1) * kHRH + S.lane + kSlots * slot_floats<LIN>();
+    S.rb = (2 * S.w + 1) * kHRH + S.lane + kSlots * Tl::kSlot;
     S.gown = (unsigned)(S.j0 + 2 * S.w) * (unsigned)N + (unsigned)(S.k0 + 2 * S.lane);
     S.smem = (unsigned)__cvta_generic_to_shared(rsm);
 #pragma unroll
-    for (int t = 0; t < kStage; ++t) {
-        const int e = tid + t * kBT;   // staged position: row rr, column k0 - 2 + q
+    for (int t = 0; t < Tl::kStage; ++t) {
+        const int e = tid + t * Tl::kBT;   // staged position: row rr, column k0 - 2 + q
         const int rr = e / kHOW, q = e - rr * kHOW;
         const unsigned so = e < kHOS ? (unsigned)(rr * kHOR + (q & 1) * kHOH + (q >> 1)) : kNoStage;
         const unsigned go = (unsigned)wrapn(S.j0 - 2 + (e < kHOS ? rr : 0), N) * (unsigned)N +
@@ -503,11 +535,14 @@ bool g_reg_ready = false;
 
 cudaError_t prepare_reg_sweeps()
 {
-    cudaError_t e = cudaFuncSetAttribute(k_sweep_reg<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)reg_smem_bytes<false>());
+    cudaError_t e = cudaFuncSetAttribute(k_sweep_reg<FAS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)Tile<FAS>::kSmem);
     if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k_sweep_reg<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)reg_smem_bytes<true>());
+        e = cudaFuncSetAttribute(k_sweep_reg<LIN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)Tile<LIN>::kSmem);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(k_sweep_reg<LIN0>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)Tile<LIN0>::kSmem);
     if (e == cudaSuccess) g_reg_ready = true;
     return e;
 }
@@ -518,7 +553,7 @@ cudaError_t prepare_reg_sweeps()
 bool reg_sweep_ok(int N, const float *src, const float *dst, const float *g, const float *th)
 {
     auto al = [](const void *p, uintptr_t a) { return p == nullptr || ((uintptr_t)p % a) == 0; };
-    return N >= kFusedMinN && N % kBK == 0 && N % kBJ == 0 && al(src, 4) && al(dst, 8) && al(g, 16) &&
+    return N >= kFusedMinN && N % kBK == 0 && al(src, 4) && al(dst, 8) && al(g, 16) &&
            al(th, 4);
 }
 
@@ -540,14 +575,17 @@ cudaError_t reg_sweep_launch(bool lin, int N, const float *src, float *dst, cons
         if (e != cudaSuccess) return e;
     }
     const int CI = reg_sweep_chunk(N, chunk);
-    const dim3 grid(N / kBK, N / kBJ, N / CI);
     note_launch();
-    if (lin)
-        k_sweep_reg<true><<<grid, kBT, reg_smem_bytes<true>(), s>>>(src, dst, g, th, cptr, cval, N, CI, ih2,
-                                                                    h2_6, rule, gshift);
+    const dim3 grid(N / kBK, N / Tile<LIN>::kBJ, N / CI);
+    if (!lin)
+        k_sweep_reg<FAS><<<grid, Tile<FAS>::kBT, Tile<FAS>::kSmem, s>>>(
+            src, dst, g, nullptr, cptr, cval, N, CI, ih2, h2_6, rule, gshift);
+    else if (src)
+        k_sweep_reg<LIN><<<grid, Tile<LIN>::kBT, Tile<LIN>::kSmem, s>>>(
+            src, dst, g, th, nullptr, 0.0, N, CI, ih2, h2_6, rule, gshift);
     else
-        k_sweep_reg<false><<<grid, kBT, reg_smem_bytes<false>(), s>>>(src, dst, g, th, cptr, cval, N, CI, ih2,
-                                                                      h2_6, rule, gshift);
+        k_sweep_reg<LIN0><<<grid, Tile<LIN0>::kBT, Tile<LIN0>::kSmem, s>>>(
+            nullptr, dst, g, th, nullptr, 0.0, N, CI, ih2, h2_6, rule, gshift);
     return cudaGetLastError();
 }
 

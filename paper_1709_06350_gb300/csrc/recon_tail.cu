@@ -21,7 +21,10 @@
 //  * Sums are double-float (48 bits) for FP32 levels, FP64 for FP64 ones: an
 //    FP64 addition holds a warp for 16 cycles of the SM's FP64 pipe, and the
 //    block sums of the coarsest solve were most of its time.
-//  * FP32 levels are relaxed two cells at a time on the paired instructions.
+//  * The linear levels are relaxed two cells at a time on the paired
+//    instructions.  The FAS levels keep the arithmetic of the grid kernels
+//    (cell_update, det_IH) operation for operation: a mixed solve's last
+//    digits follow the FP32 rounding of its FAS cycles (1e-10 of phi).
 //
 // What bounds it: latency.  One pass over 32^3 takes ~3 us, one over 4^3 ~0.5,
 // at 4-22% issue; a third of the stalls of a cold launch are instruction
@@ -59,8 +62,7 @@ __device__ __forceinline__ df acc_lane(df v, int l)
 }
 __device__ __forceinline__ double acc_lane(double v, int l) { return __shfl_sync(0xffffffffu, v, l); }
 
-// V: the type of sums; the two-cell forms of the cell arithmetic (FP32: the
-// paired instructions; FP64: one after the other, the second only if `two`)
+// V: the type of sums
 template <typename T>
 struct Math;
 template <>
@@ -84,25 +86,6 @@ struct Math<float> {
     static __device__ __forceinline__ bool le(V a, V b) { return a.hi < b.hi || (a.hi == b.hi && a.lo <= b.lo); }
     static __device__ __forceinline__ float round(V a) { return a.hi; }
     static __device__ __forceinline__ double get(V a) { return (double)a.hi + (double)a.lo; }
-    // new values va, vb of two cells with right sides ra, rb; fa, fb: their residuals
-    static __device__ __forceinline__ void update(const Nb19<float> &a, const Nb19<float> &b, float ra, float rb,
-                                                  float ih2, float h2_6, int rule, bool, float &va, float &vb,
-                                                  float &fa, float &fb)
-    {
-        float2 F;
-        const float2 v = fas_update2_det(pack19(a, b), make_float2(ra, rb), ih2, 3.0f * h2_6, h2_6, rule, &F);
-        va = v.x;
-        vb = v.y;
-        fa = -F.x;
-        fb = -F.y;
-    }
-    static __device__ __forceinline__ void det(const Nb19<float> &a, const Nb19<float> &b, float ih2, bool, float &da,
-                                               float &db)
-    {
-        const float2 d = det2(pack19(a, b), ih2);
-        da = d.x;
-        db = d.y;
-    }
 };
 template <>
 struct Math<double> {
@@ -115,19 +98,6 @@ struct Math<double> {
     static __device__ __forceinline__ bool le(V a, V b) { return a <= b; }
     static __device__ __forceinline__ double round(V a) { return a; }
     static __device__ __forceinline__ double get(V a) { return a; }
-    static __device__ __forceinline__ void update(const Nb19<double> &a, const Nb19<double> &b, double ra, double rb,
-                                                  double ih2, double h2_6, int rule, bool two, double &va, double &vb,
-                                                  double &fa, double &fb)
-    {
-        va = cell_update(a, ra, ih2, h2_6, rule, &fa);
-        if (two) vb = cell_update(b, rb, ih2, h2_6, rule, &fb);
-    }
-    static __device__ __forceinline__ void det(const Nb19<double> &a, const Nb19<double> &b, double ih2, bool two,
-                                               double &da, double &db)
-    {
-        da = det_IH(a, ih2);
-        if (two) db = det_IH(b, ih2);
-    }
 };
 
 // the dynamic shared memory
@@ -505,7 +475,8 @@ struct Tail {
     __device__ void prolong(const Level<T> &G, int fine, int cn, int co, T s) const
     {
         const int Nc = G.half, NcNc = Nc * Nc;
-        const T w0 = T(0.75), w1 = T(0.25);
+        // rounded once: a quarter of `far` is exact
+        auto mix = [](T near, T far) { return fma(T(0.75), near, T(0.25) * far); };
         parents(G, [&](int I, int J, int K, int fp) {
             const Home h = home(G.l + 1, I);
             const T *base = at(smem<T>(), h.r);
@@ -530,18 +501,18 @@ struct Tail {
 #pragma unroll
                 for (int b = 0; b < 3; ++b)
 #pragma unroll
-                    for (int c = 0; c < 3; ++c) u[b][c] = w0 * d[1][b][c] + w1 * d[ei ? 2 : 0][b][c];
+                    for (int c = 0; c < 3; ++c) u[b][c] = mix(d[1][b][c], d[ei ? 2 : 0][b][c]);
 #pragma unroll
                 for (int ej = 0; ej < 2; ++ej) {
                     T v[3];
 #pragma unroll
-                    for (int c = 0; c < 3; ++c) v[c] = w0 * u[1][c] + w1 * u[ej ? 2 : 0][c];
+                    for (int c = 0; c < 3; ++c) v[c] = mix(u[1][c], u[ej ? 2 : 0][c]);
                     Row w;
                     w.ip = fp + ei;
                     w.c = (w.ip + G.halo) * G.NN;
                     const int o = (2 * J + ej) * G.N + 2 * K;
                     const T *x = smem<T>() + fine + w.c + o;
-                    const T x0 = x[0] + s * (w0 * v[1] + w1 * v[0]), x1 = x[1] + s * (w0 * v[1] + w1 * v[2]);
+                    const T x0 = x[0] + s * mix(v[1], v[0]), x1 = x[1] + s * mix(v[1], v[2]);
                     put(G, fine, w, o, x0);
                     put(G, fine, w, o + 1, x1);
                 }
@@ -617,6 +588,9 @@ __global__ void __launch_bounds__(NT, 1) k_fas_tail(const __grid_constant__ Tail
     Tail<T, NT> C(A);
     // right side of cell k of a row, without c (g has no halos)
     auto g_at = [&](const Level<T> &G, const Row &w, int k) { return smem<T>()[C.arr(G, 3) + w.ip * G.NN + w.r + k]; };
+    auto update = [&](const Level<T> &G, int src, const Row &w, int k, T c) {
+        return cell_update(C.nb(G, src, w, k), g_at(G, w, k) + c, A.ih2[G.l], A.h2_6[G.l], A.rule);
+    };
     // snapshot red-black sweeps: t -> w (red), w -> t (black)
     auto sweeps = [&](const Level<T> &G, int count, T c) {
         const int t = C.arr(G, 0), w = C.arr(G, 1);
@@ -627,10 +601,7 @@ __global__ void __launch_bounds__(NT, 1) k_fas_tail(const __grid_constant__ Tail
                 int ra, ba, rb, bb;
                 const Row wa = C.pair(G, ia, ra, ba), wb = C.pair(G, ib, rb, bb);
                 const int ka = black ? ba : ra, kb = black ? bb : rb, oa = black ? ra : ba, ob = black ? rb : bb;
-                const Nb19<T> na = C.nb(G, src, wa, ka), nb = two ? C.nb(G, src, wb, kb) : na;
-                T va, vb, fa, fb;
-                M::update(na, nb, g_at(G, wa, ka) + c, (two ? g_at(G, wb, kb) : g_at(G, wa, ka)) + c, A.ih2[G.l],
-                          A.h2_6[G.l], A.rule, two, va, vb, fa, fb);
+                const T va = update(G, src, wa, ka, c), vb = two ? update(G, src, wb, kb, c) : va;
                 if (ona) {
                     C.put(G, dst, wa, wa.r + ka, va);
                     C.put(G, dst, wa, wa.r + oa, smem<T>()[src + wa.c + wa.r + oa]);
@@ -649,15 +620,14 @@ __global__ void __launch_bounds__(NT, 1) k_fas_tail(const __grid_constant__ Tail
         C.twos(G, G.np * G.NN, [&](int ia, int ib, bool ona, bool onb, bool two) {
             int ka, kb;
             const Row wa = C.cell(G, ia, ka), wb = C.cell(G, ib, kb);
-            const Nb19<T> na = C.nb(G, t, wa, ka), nb = two ? C.nb(G, t, wb, kb) : na;
-            T da, db;
-            M::det(na, nb, A.ih2[G.l], two, da, db);
+            const T da = det_IH(C.nb(G, t, wa, ka), A.ih2[G.l]);
+            const T db = two ? det_IH(C.nb(G, t, wb, kb), A.ih2[G.l]) : da;
             if (ona) f(wa, ka, da);
             if (onb) f(wb, kb, db);
         });
     };
     // the right side det(I + H R theta) + s (R r - mean R r) of a level from
-    // its theta, R r in g and the sum of R r; s and 1 / s as in k_finalize_scale
+    // its theta, R r in g and the sum of R r; s and 1 / s as in k_coarse_rhs
     auto form = [&](const Level<T> &G, V sum) {
         const int w = C.arr(G, 1), g = C.arr(G, 3);
         const V mean = M::mul(sum, A.rn[G.l]);
@@ -746,20 +716,17 @@ __global__ void __launch_bounds__(NT, 1) k_fas_tail(const __grid_constant__ Tail
         C.coarsest(
             G, C.arr(G, 0), C.arr(G, 1), C.arr(G, 3) + C.own(G),
             [&](int src, const Row &w, int kr, int kb, T &rr, T &rb) {
-                const Nb19<T> a = C.nb(G, src, w, kr), b = C.nb(G, src, w, kb);
-                const T ga = g_at(G, w, kr) + c, gb = g_at(G, w, kb) + c;
-                T va, vb;
-                M::update(a, b, ga, gb, A.ih2[G.l], A.h2_6[G.l], A.rule, false, va, vb, rr, rb);
-                if constexpr (sizeof(T) == 8) rb = gb - det_IH(b, A.ih2[G.l]);
-                return va;
+                rb = (g_at(G, w, kb) + c) - det_IH(C.nb(G, src, w, kb), A.ih2[G.l]);
+                if constexpr (sizeof(T) == 8) {
+                    return cell_update(C.nb(G, src, w, kr), g_at(G, w, kr) + c, A.ih2[G.l], A.h2_6[G.l], A.rule, &rr);
+                } else {
+                    rr = (g_at(G, w, kr) + c) - det_IH(C.nb(G, src, w, kr), A.ih2[G.l]);
+                    // (loaded again: shared products would round differently than in cell_update alone)
+                    asm volatile("" ::: "memory");
+                    return update(G, src, w, kr, c);
+                }
             },
-            [&](int src, const Row &w, int kb) {
-                const Nb19<T> a = C.nb(G, src, w, kb);
-                const T ga = g_at(G, w, kb) + c;
-                T va, vb, fa, fb;
-                M::update(a, a, ga, ga, A.ih2[G.l], A.h2_6[G.l], A.rule, false, va, vb, fa, fb);
-                return va;
-            });
+            [&](int src, const Row &w, int kb) { return update(G, src, w, kb, c); });
     }
     // up: the corrections and post-smoothing
     for (int l = nl - 2; l >= 0; --l) {
