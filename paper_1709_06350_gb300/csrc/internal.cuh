@@ -49,7 +49,7 @@ struct recon_handle {
     double *t64[kMaxLevels] = {}, *g64[kMaxLevels] = {}, *told64[kMaxLevels] = {},
            *aux64[kMaxLevels] = {};
     double *work64 = nullptr;    // N^3: smoother ping-pong, displace numerator
-    double *work64b = nullptr;   // N^3: displace denominator, adjoint scratch
+    double *work64b = nullptr;   // N^3: FP64 displacement sums, adjoint scratch
 
     // FP32 hierarchy (MIXED): FAS theta / g / saved theta / aux, linear e / f.
     float *t32[kMaxLevels] = {}, *g32[kMaxLevels] = {}, *told32[kMaxLevels] = {},
@@ -191,10 +191,7 @@ cudaError_t gaussianise(recon_handle *H, const double *v, size_t n, double *g);
 cudaError_t smooth_density(int N, double L, double R, double floor_, const double *rho, double *b, float *w32,
                            double *mean, cudaStream_t s);
 
-// phi -> (hi, lo) FP32 parts (recon_mg.cu)
-__global__ void k_split_df(const double *__restrict__ a, float *__restrict__ hi, float *__restrict__ lo,
-                           size_t n);
 cudaError_t displace(int N, double L, const double *phi, const double *b, double *psi,
-                     double *deltaL, double *scratch, double *split, cudaStream_t s);
+                     double *deltaL, double *scratch, cudaStream_t s);
 
 }  // namespace recon

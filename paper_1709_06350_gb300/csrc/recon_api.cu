@@ -380,7 +380,7 @@ recon_status recon_displace(recon_handle *H, const double *phi, const double *b,
     if (!phi || !b || !psi || !deltaL) return set_err(H, RECON_E_INVALID, "NULL pointer");
     if (!gpu_reachable(psi) || !gpu_reachable(deltaL))
         return set_err(H, RECON_E_INVALID, "psi and deltaL must be device or page-locked host memory");
-    return cuda_status(H, displace(H->N, H->L, phi, b, psi, deltaL, H->work64, H->work64b, H->stream),
+    return cuda_status(H, displace(H->N, H->L, phi, b, psi, deltaL, H->work64, H->stream),
                        "displace");
 }
 
