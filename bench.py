@@ -1078,33 +1078,23 @@ FP64_FLOPS_PER_CELL_UPDATE = 70.0
 
 
 def fp64_rooflines(recon, torch, N, L, dev, stream):
-    """The FP64 path's smoother at N^3 against the measured FP64 FMA rate:
-    the fused sweep (both colours, one launch) and the two-pass kernels (an
-    array not aligned to an element pair runs them: two launches a sweep)."""
+    """The FP64 path's smoother at N^3 (two launches a sweep) against the
+    measured FP64 FMA rate."""
     from paper_1709_06350_gb300 import synth
     peak = fp64_peak_tflops(recon, torch, dev, stream)
     h = L / N
     th = torch.from_numpy(synth.smooth_field(N, 1, 0.3 * h * h, kmax=4)).to(dev, torch.float64)
     g = torch.from_numpy(1.0 + synth.smooth_field(N, 2, 0.4, kmax=4)).to(dev, torch.float64)
     work = torch.empty_like(th)
-    t_fused = _time_launches(torch, stream, lambda k: recon.recon_step_sweep(
+    t = _time_launches(torch, stream, lambda k: recon.recon_step_sweep(
         th, g, 0.0, h, sweeps=k, work=work, stream=stream), 3)
-    buf = torch.empty(th.numel() + 1, dtype=torch.float64, device=dev)
-    tu = buf[1:].view(th.shape)
-    tu.copy_(th)
-    t_two = _time_launches(torch, stream, lambda k: recon.recon_step_sweep(
-        tu, g, 0.0, h, sweeps=k, work=work, stream=stream), 3)
-    del th, g, work, buf, tu
-    out = []
-    for name, t, launches in (("k_sweep_fused<double, FAS> (FP64 red-black Newton smoother, one fused sweep)",
-                               t_fused, 1),
-                              ("k_rb_pass<double> (FP64 red-black Newton smoother, one colour pass)", t_two, 2)):
-        flops = FP64_FLOPS_PER_CELL_UPDATE * N ** 3 / launches
-        ach = flops / (t / launches) / 1e12
-        out.append({"kernel": name, "bound": "fp64", "achieved": ach, "peak": peak, "unit": "TFLOP/s",
-                    "frac": ach / peak, "peak_source": "measured: recon_measure_fp64_fma (FP64 FMA chains)",
-                    "algorithmic_flops_per_launch": flops, "avg_launch_ms": t / launches * 1e3})
-    return out
+    del th, g, work
+    flops, launches = FP64_FLOPS_PER_CELL_UPDATE * N ** 3 / 2, 2
+    ach = flops / (t / launches) / 1e12
+    return [{"kernel": "k_rb_pass<double> (FP64 red-black Newton smoother, one colour pass)", "bound": "fp64",
+             "achieved": ach, "peak": peak, "unit": "TFLOP/s", "frac": ach / peak,
+             "peak_source": "measured: recon_measure_fp64_fma (FP64 FMA chains)",
+             "algorithmic_flops_per_launch": flops, "avg_launch_ms": t / launches * 1e3}]
 
 
 if __name__ == "__main__":
