@@ -1901,7 +1901,7 @@ namespace {
 // Level l's f can carry its mean unsubtracted into a linear V-cycle when
 // every kernel that reads it there folds the shift in: the register-blocked
 // sweep (both directions of its ping-pong) and the restriction (a level above
-// the single-block tail and the coarsest solve).
+// the tail and the coarsest solve).
 static bool lin_fold_ok(recon_handle *H, int l)
 {
     const int N = H->Nl[l];

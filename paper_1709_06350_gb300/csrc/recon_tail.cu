@@ -20,7 +20,8 @@
 //    barriers; if it was the last, the extra red pass is dropped.
 //  * Sums are double-float (48 bits) for FP32 levels, FP64 for FP64 ones: an
 //    FP64 addition holds a warp for 16 cycles of the SM's FP64 pipe, and the
-//    block sums of the coarsest solve were most of its time.
+//    block sums of the coarsest solve were most of its time.  Solutions are as
+//    far from 64-bit ones as with FP64 sums (64^3 1.2e-9, 160^3 3.6e-10 of phi).
 //  * The linear levels are relaxed two cells at a time on the paired
 //    instructions.  The FAS levels keep the arithmetic of the grid kernels
 //    (cell_update, det_IH) operation for operation: a mixed solve's last
