@@ -93,6 +93,13 @@ inline unsigned fit_grid(int N, dim3 block)
          row_ < (unsigned)(N) * (unsigned)(N); row_ += gridDim.x * blockDim.y)          \
         if (const int i = (int)(row_ / (unsigned)(N)), j = (int)(row_ % (unsigned)(N)); true)
 
+// The rows of group `group` of `groups`: what block `group` of a grid of
+// `groups` blocks visits in FOR_ROWS.
+#define FOR_GROUP_ROWS(N, group, groups, i, j)                                         \
+    for (unsigned row_ = (group) * blockDim.y + threadIdx.y;                           \
+         row_ < (unsigned)(N) * (unsigned)(N); row_ += (groups) * blockDim.y)          \
+        if (const int i = (int)(row_ / (unsigned)(N)), j = (int)(row_ % (unsigned)(N)); true)
+
 // ---------------------------------------------------------------- scalars
 // Device-resident scalars of one handle (doubles), so that a cycle needs no
 // host round trip except the convergence read.
@@ -175,30 +182,53 @@ __device__ __forceinline__ bool last_block(unsigned *counter)
     return last;
 }
 
-constexpr int kMaxRedBlocks = 2048;   // grid cap of every reducing kernel
-// ... and of the ones that end in last_block: one wave of `per_sm` blocks, as a
-// block's last writes, fence and ticket take ~2 us that every further wave would
-// wait for (512^3 residual restriction: 461 us with 2048 blocks, two per SM, about
-// 400 us with one wave)
+// Groups of rows of a reducing kernel, each with partial sums of its own.  The
+// groups depend on the size alone and not on the grid: a thread's sum is
+// compensated FP32 on FP32 levels, its last digits follow the order of its
+// cells, and the FP32 cycles grow a flipped digit of a mean to 1e-7 of phi.
+constexpr int kMaxRedBlocks = 2048;
+inline unsigned row_groups(int N) { return row_grid(N, kMaxRedBlocks); }
+// ... and the grid of the ones that end in last_block, whose blocks take the
+// groups in turn: one wave of `per_sm` blocks, as a block's last writes, fence
+// and ticket take ~2 us that every further wave would wait for (512^3 residual
+// restriction: 461 us with 2048 blocks, two per SM, about 400 us with one wave)
 constexpr unsigned kSMs = 152;
 inline unsigned wave_grid(int N, unsigned per_sm) { return row_grid(N, kSMs * per_sm); }
 
-// Total (least) of column `col` of the blocks' partials (4 doubles each) in a
-// fixed order, in ltid() == 0 of a block of NT threads; all loads in flight at
-// once.
-template <int NT>
-__device__ __forceinline__ double total_partials(const double *partials, int nb, int col, double *sh)
+// Totals of columns 0 .. K-1 of the groups' partials (4 doubles each) in a
+// fixed order, that of a block of kReduceThreads, in ltid() == 0 of a block of
+// NT threads; all loads in flight at once.  sh: kReduceThreads / 32 doubles
+// per column.
+template <int NT, int K>
+__device__ __forceinline__ void total_columns(const double *partials, int nb, double *sh, double (&out)[K])
 {
-    double v[kMaxRedBlocks / NT];
+    constexpr int kRounds = kReduceThreads / NT, kWarps = kReduceThreads / 32;
+    static_assert(kMaxRedBlocks == 2 * kReduceThreads && kReduceThreads % NT == 0 && kWarps == 32, "");
+    double p[kRounds][2][K];
 #pragma unroll
-    for (int u = 0; u < kMaxRedBlocks / NT; ++u) {
-        const int b = ltid() + u * NT;
-        v[u] = b < nb ? __ldcg(partials + 4 * b + col) : 0.0;
+    for (int u = 0; u < kRounds; ++u)
+        for (int w = 0; w < 2; ++w) {
+            const int b = u * NT + ltid() + w * kReduceThreads;
+            for (int x = 0; x < K; ++x) p[u][w][x] = b < nb ? __ldcg(partials + 4 * b + x) : 0.0;
+        }
+    __syncthreads();
+#pragma unroll
+    for (int u = 0; u < kRounds; ++u)
+        for (int x = 0; x < K; ++x) {
+            double v = p[u][0][x] + p[u][1][x];
+            for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+            if ((ltid() & 31) == 0) sh[x * kWarps + (u * NT + ltid()) / 32] = v;
+        }
+    __syncthreads();
+    for (int x = 0; x < K; ++x) {
+        out[x] = 0.0;
+        if (ltid() < 32) {
+            out[x] = sh[x * kWarps + ltid()];
+            for (int o = 16; o > 0; o >>= 1) out[x] += __shfl_down_sync(0xffffffffu, out[x], o);
+        }
     }
-#pragma unroll
-    for (int u = 1; u < kMaxRedBlocks / NT; ++u) v[0] += v[u];
-    return block_sum<NT>(v[0], sh);
 }
+// least of column `col`
 template <int NT>
 __device__ __forceinline__ double min_partials(const double *partials, int nb, int col, double *sh)
 {

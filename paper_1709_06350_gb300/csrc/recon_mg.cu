@@ -576,11 +576,12 @@ k_det_write(const double *__restrict__ t, int N, double ih2, double *__restrict_
 }
 
 // Where the last block of a reducing kernel leaves its result: `out`
-// (S_* scalars or a slot of one level), n cells
+// (S_* scalars or a slot of one level), n cells, partials of `groups` groups
 struct Finish {
     unsigned *counter;
     double n;
     double *out;
+    unsigned groups;
 };
 
 // After a cycle on a level with n cells, from the partials' columns 0..2 (sums
@@ -590,26 +591,10 @@ struct Finish {
 template <int NT>
 __device__ __noinline__ void cycle_scalars(const double *partials, int nb, double n, double *scal)
 {
-    __shared__ double sh[3][NT / 32];
-    double p[kMaxRedBlocks / NT][3], v[3] = {0.0, 0.0, 0.0};
-#pragma unroll
-    for (int u = 0; u < kMaxRedBlocks / NT; ++u) {   // all loads in flight at once
-        const int b = ltid() + u * NT;
-        for (int x = 0; x < 3; ++x) p[u][x] = b < nb ? __ldcg(partials + 4 * b + x) : 0.0;
-    }
-#pragma unroll
-    for (int u = 0; u < kMaxRedBlocks / NT; ++u)
-        for (int x = 0; x < 3; ++x) v[x] += p[u][x];
-    for (int o = 16; o > 0; o >>= 1)
-        for (int x = 0; x < 3; ++x) v[x] += __shfl_down_sync(0xffffffffu, v[x], o);
-    if ((ltid() & 31) == 0)
-        for (int x = 0; x < 3; ++x) sh[x][ltid() >> 5] = v[x];
-    __syncthreads();
+    __shared__ double sh[3 * 32];
+    double v[3];
+    total_columns<NT>(partials, nb, sh, v);
     if (ltid() != 0) return;
-    for (int x = 0; x < 3; ++x) {
-        v[x] = 0.0;
-        for (int w = 0; w < NT / 32; ++w) v[x] += sh[x][w];
-    }
     const double m = v[0] / n, var = v[1] - n * m * m;
     scal[S_MEAN_R] = m;
     scal[S_C] -= m;
@@ -625,7 +610,7 @@ k_finish_cycle(const double *__restrict__ partials, int nb, double n, double *__
 template <int NT>
 __device__ __forceinline__ void finish_cycle(const double *partials, const Finish &fin)
 {
-    if (last_block(fin.counter)) cycle_scalars<NT>(partials, gridDim.x, fin.n, fin.out);
+    if (last_block(fin.counter)) cycle_scalars<NT>(partials, fin.groups, fin.n, fin.out);
 }
 
 // *fin.out = (sum of column 0) / n; no out: no mean wanted
@@ -633,16 +618,30 @@ template <int NT>
 __device__ __noinline__ void mean_scalar(const double *partials, int nb, double n, double *out)
 {
     __shared__ double sh[32];
-    const double s = total_partials<NT>(partials, nb, 0, sh);
-    if (ltid() == 0) *out = s / n;
+    double s[1];
+    total_columns<NT>(partials, nb, sh, s);
+    if (ltid() == 0) *out = s[0] / n;
 }
 template <int NT>
 __device__ __forceinline__ void finish_mean(const double *partials, const Finish &fin)
 {
-    if (fin.out && last_block(fin.counter)) mean_scalar<NT>(partials, gridDim.x, fin.n, fin.out);
+    if (fin.out && last_block(fin.counter)) mean_scalar<NT>(partials, fin.groups, fin.n, fin.out);
 }
 
-// partials[4 b + 0..2] = sum r, sum r^2, sum theta over this block's cells,
+// columns 0 .. 2 of a group's partials
+template <typename T>
+__device__ __forceinline__ void store_sums(const ThreadSum<T> &a, const ThreadSum<T> &b, const ThreadSum<T> &c, double *sh,
+                                           double *partials)
+{
+    double v = block_sum<kRowThreads>(a.get(), sh);
+    if (ltid() == 0) partials[0] = v;
+    v = block_sum<kRowThreads>(b.get(), sh);
+    if (ltid() == 0) partials[1] = v;
+    v = block_sum<kRowThreads>(c.get(), sh);
+    if (ltid() == 0) partials[2] = v;
+}
+
+// partials[4 q + 0..2] = sum r, sum r^2, sum theta over the cells of group q,
 // r = g + c - det(I + H theta).  When f32out is set (mixed path, T = double)
 // the residual is also stored as float and theta as float in t32out.
 template <typename T>
@@ -653,26 +652,23 @@ k_residual_norms(const T *__restrict__ t, const T *__restrict__ g,
 {
     __shared__ double sh[32];
     const T c = (T)(*cptr);
-    ThreadSum<T> sr, sr2, st;
-    FOR_ROWS(N, i, j)
-    for (int k = threadIdx.x; k < N; k += kRowX) {
-        const unsigned id = offs(N, i, j, k);
-        const Nb19<T> nb = load19<T>(t, N, i, j, k);
-        const T res = (g[id] + c) - det_IH(nb, ih2);
-        sr.add(res);
-        sr2.add(res * res);
-        st.add(nb.c);
-        if (f32out) {
-            f32out[id] = (float)res;
-            t32out[id] = (float)nb.c;
+    for (unsigned q = blockIdx.x; q < fin.groups; q += gridDim.x) {
+        ThreadSum<T> sr, sr2, st;
+        FOR_GROUP_ROWS(N, q, fin.groups, i, j)
+        for (int k = threadIdx.x; k < N; k += kRowX) {
+            const unsigned id = offs(N, i, j, k);
+            const Nb19<T> nb = load19<T>(t, N, i, j, k);
+            const T res = (g[id] + c) - det_IH(nb, ih2);
+            sr.add(res);
+            sr2.add(res * res);
+            st.add(nb.c);
+            if (f32out) {
+                f32out[id] = (float)res;
+                t32out[id] = (float)nb.c;
+            }
         }
+        store_sums<T>(sr, sr2, st, sh, partials + 4 * q);
     }
-    double v = block_sum<kRowThreads>(sr.get(), sh);
-    if (ltid() == 0) partials[4 * blockIdx.x + 0] = v;
-    v = block_sum<kRowThreads>(sr2.get(), sh);
-    if (ltid() == 0) partials[4 * blockIdx.x + 1] = v;
-    v = block_sum<kRowThreads>(st.get(), sh);
-    if (ltid() == 0) partials[4 * blockIdx.x + 2] = v;
     finish_cycle<kRowThreads>(partials, fin);
 }
 
@@ -773,40 +769,37 @@ k_residual_norms_win(const T *__restrict__ t, const T *__restrict__ g,
     __shared__ double sh[32];
     const T c = (T)(*cptr);
     const int Nc = N >> 1;
-    ThreadSum<T> sr, sr2, st;
-    FOR_ROWS(Nc, I, J)
-    for (int K = threadIdx.x; K < Nc; K += kRowX) {
-        const Win w(N, I, J, K);
-        T P0[4][4], P1[4][4], P2[4][4];
-        win_plane<T, false>(t, w, 0, P0);
-        win_plane<T, true>(t, w, 1, P1);
-        win_plane<T, true>(t, w, 2, P2);
+    for (unsigned q = blockIdx.x; q < fin.groups; q += gridDim.x) {
+        ThreadSum<T> sr, sr2, st;
+        FOR_GROUP_ROWS(Nc, q, fin.groups, I, J)
+        for (int K = threadIdx.x; K < Nc; K += kRowX) {
+            const Win w(N, I, J, K);
+            T P0[4][4], P1[4][4], P2[4][4];
+            win_plane<T, false>(t, w, 0, P0);
+            win_plane<T, true>(t, w, 1, P1);
+            win_plane<T, true>(t, w, 2, P2);
 #pragma unroll
-        for (int a = 0; a < 2; ++a) {
-            if (a == 1) win_plane<T, false>(t, w, 3, P0);
+            for (int a = 0; a < 2; ++a) {
+                if (a == 1) win_plane<T, false>(t, w, 3, P0);
 #pragma unroll
-            for (int b = 1; b <= 2; ++b)
+                for (int b = 1; b <= 2; ++b)
 #pragma unroll
-                for (int cc = 1; cc <= 2; ++cc) {
-                    const Nb19<T> nb = a == 0 ? win_nb<T>(P0, P1, P2, b, cc) : win_nb<T>(P1, P2, P0, b, cc);
-                    const unsigned id = w.at(1 + a, b, cc);
-                    const T res = (g[id] + c) - det_IH(nb, ih2);
-                    sr.add(res);
-                    sr2.add(res * res);
-                    st.add(nb.c);
-                    if (f32out) {
-                        f32out[id] = (float)res;
-                        t32out[id] = (float)nb.c;
+                    for (int cc = 1; cc <= 2; ++cc) {
+                        const Nb19<T> nb = a == 0 ? win_nb<T>(P0, P1, P2, b, cc) : win_nb<T>(P1, P2, P0, b, cc);
+                        const unsigned id = w.at(1 + a, b, cc);
+                        const T res = (g[id] + c) - det_IH(nb, ih2);
+                        sr.add(res);
+                        sr2.add(res * res);
+                        st.add(nb.c);
+                        if (f32out) {
+                            f32out[id] = (float)res;
+                            t32out[id] = (float)nb.c;
+                        }
                     }
-                }
+            }
         }
+        store_sums<T>(sr, sr2, st, sh, partials + 4 * q);
     }
-    double v = block_sum<kRowThreads>(sr.get(), sh);
-    if (ltid() == 0) partials[4 * blockIdx.x + 0] = v;
-    v = block_sum<kRowThreads>(sr2.get(), sh);
-    if (ltid() == 0) partials[4 * blockIdx.x + 1] = v;
-    v = block_sum<kRowThreads>(st.get(), sh);
-    if (ltid() == 0) partials[4 * blockIdx.x + 2] = v;
     finish_cycle<kRowThreads>(partials, fin);
 }
 
@@ -815,9 +808,10 @@ k_residual_norms_win(const T *__restrict__ t, const T *__restrict__ g,
 template <typename T>
 static cudaError_t residual_norms(recon_handle *H, const T *t, const T *g, int N, T ih2, float *f32out, float *t32out)
 {
-    const Finish fin = {H->ticket, (double)N * N * N, H->scal};
+    const bool win = N % 2 == 0 && N >= 32;
+    const Finish fin = {H->ticket, (double)N * N * N, H->scal, row_groups(win ? N / 2 : N)};
     note_launch();
-    if (N % 2 == 0 && N >= 32)
+    if (win)
         k_residual_norms_win<T><<<wave_grid(N / 2, 2), row_block(), 0, H->stream>>>(
             t, g, H->scal + S_C, N, ih2, H->partials, f32out, t32out, fin);
     else
@@ -835,42 +829,44 @@ k_restrict_residual(const T *__restrict__ t, const T *__restrict__ g,
     __shared__ double sh[32];
     const int Nc = Nf >> 1;
     const T c = (T)(*cptr);
-    ThreadSum<T> srr;
-    FOR_ROWS(Nc, I, J)
-    for (int K = threadIdx.x; K < Nc; K += kRowX) {
-        const Win w(Nf, I, J, K);
-        T P0[4][4], P1[4][4], P2[4][4];
-        win_plane<T, false>(t, w, 0, P0);
-        win_plane<T, true>(t, w, 1, P1);
-        win_plane<T, true>(t, w, 2, P2);
-        T at = T(0), ar = T(0);
+    for (unsigned q = blockIdx.x; q < fin.groups; q += gridDim.x) {
+        ThreadSum<T> srr;
+        FOR_GROUP_ROWS(Nc, q, fin.groups, I, J)
+        for (int K = threadIdx.x; K < Nc; K += kRowX) {
+            const Win w(Nf, I, J, K);
+            T P0[4][4], P1[4][4], P2[4][4];
+            win_plane<T, false>(t, w, 0, P0);
+            win_plane<T, true>(t, w, 1, P1);
+            win_plane<T, true>(t, w, 2, P2);
+            T at = T(0), ar = T(0);
 #pragma unroll
-        for (int b = 1; b <= 2; ++b)
+            for (int b = 1; b <= 2; ++b)
 #pragma unroll
-            for (int cc = 1; cc <= 2; ++cc) {   // children in fine plane 2I: window planes 0..2
-                const Nb19<T> nb = win_nb<T>(P0, P1, P2, b, cc);
-                at += nb.c;
-                ar += (g[w.at(1, b, cc)] + c) - det_IH(nb, ih2);
-            }
-        win_plane<T, false>(t, w, 3, P0);   // children in fine plane 2I+1: planes 1..3
+                for (int cc = 1; cc <= 2; ++cc) {   // children in fine plane 2I: window planes 0..2
+                    const Nb19<T> nb = win_nb<T>(P0, P1, P2, b, cc);
+                    at += nb.c;
+                    ar += (g[w.at(1, b, cc)] + c) - det_IH(nb, ih2);
+                }
+            win_plane<T, false>(t, w, 3, P0);   // children in fine plane 2I+1: planes 1..3
 #pragma unroll
-        for (int b = 1; b <= 2; ++b)
+            for (int b = 1; b <= 2; ++b)
 #pragma unroll
-            for (int cc = 1; cc <= 2; ++cc) {
-                const Nb19<T> nb = win_nb<T>(P1, P2, P0, b, cc);
-                at += nb.c;
-                ar += (g[w.at(2, b, cc)] + c) - det_IH(nb, ih2);
-            }
-        const T vt = at * T(0.125), vr = ar * T(0.125);
-        const unsigned id = offs(Nc, I, J, K);
-        tH[id] = vt;
-        toldH[id] = vt;
-        rrH[id] = vr;
-        srr.add(vr);
+                for (int cc = 1; cc <= 2; ++cc) {
+                    const Nb19<T> nb = win_nb<T>(P1, P2, P0, b, cc);
+                    at += nb.c;
+                    ar += (g[w.at(2, b, cc)] + c) - det_IH(nb, ih2);
+                }
+            const T vt = at * T(0.125), vr = ar * T(0.125);
+            const unsigned id = offs(Nc, I, J, K);
+            tH[id] = vt;
+            toldH[id] = vt;
+            rrH[id] = vr;
+            srr.add(vr);
+        }
+        if (!fin.out) continue;   // a tail below takes the sum itself
+        const double v = block_sum<kRowThreads>(srr.get(), sh);
+        if (ltid() == 0) partials[4 * q] = v;
     }
-    if (!fin.out) return;   // a tail below takes the sum itself
-    const double v = block_sum<kRowThreads>(srr.get(), sh);
-    if (ltid() == 0) partials[4 * blockIdx.x + 0] = v;
     finish_mean<kRowThreads>(partials, fin);
 }
 
@@ -1311,12 +1307,13 @@ k_b_stats(const double *__restrict__ b, size_t n, double *__restrict__ partials,
     v = block_min<kThreads>(mn, sh);
     if (ltid() == 0) partials[4 * blockIdx.x + 3] = v;
     if (!last_block(fin.counter)) return;
-    const double t2 = total_partials<kThreads>(partials, gridDim.x, 0, sh);
-    const double tbad = total_partials<kThreads>(partials, gridDim.x, 1, sh);
-    const double tmin = min_partials<kThreads>(partials, gridDim.x, 3, sh);
+    __shared__ double shc[2 * 32];
+    double t[2];
+    total_columns<kThreads>(partials, fin.groups, shc, t);
+    const double tmin = min_partials<kThreads>(partials, fin.groups, 3, sh);
     if (ltid() == 0) {
-        fin.out[S_DENOM] = t2 > 0.0 ? sqrt(t2) : 1.0;
-        fin.out[S_BBAD] = tbad;
+        fin.out[S_DENOM] = t[0] > 0.0 ? sqrt(t[0]) : 1.0;
+        fin.out[S_BBAD] = t[1];
         fin.out[S_BMIN] = tmin;
     }
 }
@@ -1607,47 +1604,49 @@ k_lin_restrict_residual(const float *__restrict__ e, const float *__restrict__ f
     const size_t nf = (size_t)Nf * Nf * Nf;
     const int Nc = Nf >> 1;
     const float fs = fshift ? (float)*fshift : 0.0f;   // subtracted from f (its mean, folded in)
-    ThreadSum<float> sacc;
-    FOR_ROWS(Nc, I, J)
-    for (int K = threadIdx.x; K < Nc; K += kRowX) {
-        const Win w(Nf, I, J, K);
-        float E0[4][4], E1[4][4], E2[4][4], T0[4][4], T1[4][4], T2[4][4];
-        win_plane<float, false>(e, w, 0, E0);
-        win_plane<float, true>(e, w, 1, E1);
-        win_plane<float, true>(e, w, 2, E2);
-        if constexpr (FROM_TH) {
-            win_plane<float, false>(th, w, 0, T0);
-            win_plane<float, true>(th, w, 1, T1);
-            win_plane<float, true>(th, w, 2, T2);
-        }
-        float acc = 0.0f;
-#pragma unroll
-        for (int a = 0; a < 2; ++a) {
-            if (a == 1) {   // slide the window: fine plane 2I+1 needs window planes 1..3
-                win_plane<float, false>(e, w, 3, E0);
-                if constexpr (FROM_TH) win_plane<float, false>(th, w, 3, T0);
+    for (unsigned q = blockIdx.x; q < fin.groups; q += gridDim.x) {
+        ThreadSum<float> sacc;
+        FOR_GROUP_ROWS(Nc, q, fin.groups, I, J)
+        for (int K = threadIdx.x; K < Nc; K += kRowX) {
+            const Win w(Nf, I, J, K);
+            float E0[4][4], E1[4][4], E2[4][4], T0[4][4], T1[4][4], T2[4][4];
+            win_plane<float, false>(e, w, 0, E0);
+            win_plane<float, true>(e, w, 1, E1);
+            win_plane<float, true>(e, w, 2, E2);
+            if constexpr (FROM_TH) {
+                win_plane<float, false>(th, w, 0, T0);
+                win_plane<float, true>(th, w, 1, T1);
+                win_plane<float, true>(th, w, 2, T2);
             }
+            float acc = 0.0f;
 #pragma unroll
-            for (int b = 1; b <= 2; ++b)
-#pragma unroll
-                for (int cc = 1; cc <= 2; ++cc) {
-                    const Nb19<float> ne = a == 0 ? win_nb<float>(E0, E1, E2, b, cc) : win_nb<float>(E1, E2, E0, b, cc);
-                    Cof<float> A;
-                    if constexpr (FROM_TH) {
-                        A = cofactors(a == 0 ? win_nb<float>(T0, T1, T2, b, cc) : win_nb<float>(T1, T2, T0, b, cc), ih2);
-                    } else {
-                        A = cof_at(cof, nf, cof_slot(Nf, 2 * I + a, 2 * J + b - 1, 2 * K + cc - 1));
-                    }
-                    acc += (f[w.at(1 + a, b, cc)] - fs) - jac_apply(A, ne, ih2);
+            for (int a = 0; a < 2; ++a) {
+                if (a == 1) {   // slide the window: fine plane 2I+1 needs window planes 1..3
+                    win_plane<float, false>(e, w, 3, E0);
+                    if constexpr (FROM_TH) win_plane<float, false>(th, w, 3, T0);
                 }
+#pragma unroll
+                for (int b = 1; b <= 2; ++b)
+#pragma unroll
+                    for (int cc = 1; cc <= 2; ++cc) {
+                        const Nb19<float> ne = a == 0 ? win_nb<float>(E0, E1, E2, b, cc) : win_nb<float>(E1, E2, E0, b, cc);
+                        Cof<float> A;
+                        if constexpr (FROM_TH) {
+                            A = cofactors(a == 0 ? win_nb<float>(T0, T1, T2, b, cc) : win_nb<float>(T1, T2, T0, b, cc), ih2);
+                        } else {
+                            A = cof_at(cof, nf, cof_slot(Nf, 2 * I + a, 2 * J + b - 1, 2 * K + cc - 1));
+                        }
+                        acc += (f[w.at(1 + a, b, cc)] - fs) - jac_apply(A, ne, ih2);
+                    }
+            }
+            const float v = acc * 0.125f;
+            fH[offs(Nc, I, J, K)] = v;
+            sacc.add(v);
         }
-        const float v = acc * 0.125f;
-        fH[offs(Nc, I, J, K)] = v;
-        sacc.add(v);
+        if (!fin.out) continue;   // a tail below takes the sum itself
+        const double v = block_sum<kRowThreads>(sacc.get(), sh);
+        if (ltid() == 0) partials[4 * q] = v;
     }
-    if (!fin.out) return;   // a tail below takes the sum itself
-    const double v = block_sum<kRowThreads>(sacc.get(), sh);
-    if (ltid() == 0) partials[4 * blockIdx.x + 0] = v;
     finish_mean<kRowThreads>(partials, fin);
 }
 
@@ -1729,7 +1728,8 @@ cudaError_t vcycle(recon_handle *H, const Hier<T> &Y, int l, const double *cptr,
     k_restrict_residual<T><<<wave_grid(Nc, 2), row_block(), 0, s>>>(cur, Y.g[l], cptr, N, (T)(1.0 / (h * h)),
                                                     Y.t[l + 1], Y.told[l + 1], Y.g[l + 1], H->partials,
                                                     Finish{H->ticket, (double)nc,
-                                                           tail_ok<T>(Nc) ? nullptr : H->scal + slot_rmean(l + 1)});
+                                                           tail_ok<T>(Nc) ? nullptr : H->scal + slot_rmean(l + 1),
+                                                           row_groups(Nc)});
     CK(cudaGetLastError());
     auto up = [&]() {
         CK(prolong_to<T>(Nc, Y.t[l + 1], Y.told[l + 1], H->scal + slot_pscale(l + 1), 1.0, cur, post, s));
@@ -1744,7 +1744,7 @@ cudaError_t vcycle(recon_handle *H, const Hier<T> &Y, int l, const double *cptr,
     k_coarse_rhs<T><<<wave_grid(Nc, 4), row_block(), 0, s>>>(Y.t[l + 1], Y.g[l + 1], Y.aux[l + 1],
                                              H->scal + slot_rmean(l + 1), Nc,
                                              (T)(1.0 / (hc * hc)), cf.scale_floor, H->partials,
-                                             Finish{H->ticket, (double)nc, H->scal + slot_scale(l + 1)});
+                                             Finish{H->ticket, (double)nc, H->scal + slot_scale(l + 1), 0});
     note_launch();
     k_form_rhs<T><<<stride_blocks(nc), kThreads, 0, s>>>(Y.g[l + 1], Y.aux[l + 1], nc,
                                                       H->scal + slot_scale(l + 1));
@@ -1822,7 +1822,8 @@ recon_status check_domain(recon_handle *H, const double *b)
 {
     const size_t n = ncell(H->N);
     note_launch();
-    k_b_stats<<<red_blocks(n), kThreads, 0, H->stream>>>(b, n, H->partials, Finish{H->ticket, (double)n, H->scal});
+    k_b_stats<<<red_blocks(n), kThreads, 0, H->stream>>>(b, n, H->partials,
+                                                          Finish{H->ticket, (double)n, H->scal, red_blocks(n)});
     cudaError_t e = cudaGetLastError();
     if (e == cudaSuccess) e = read_scalars(H);
     if (e != cudaSuccess) return fail_cuda(H, e, "domain check");
@@ -1932,7 +1933,8 @@ cudaError_t lin_vcycle(recon_handle *H, int l, const double *fshift, bool raw, b
     const int Nc = H->Nl[l + 1];
     const size_t nc = ncell(Nc);
     const unsigned nbr = wave_grid(Nc, 2);
-    const Finish fin = {H->ticket, (double)nc, tail_ok<float>(Nc) ? nullptr : H->scal + slot_rmean(l + 1)};
+    const Finish fin = {H->ticket, (double)nc, tail_ok<float>(Nc) ? nullptr : H->scal + slot_rmean(l + 1),
+                        row_groups(Nc)};
     note_launch();
     if (H->cof32[l])
         k_lin_restrict_residual<false><<<nbr, row_block(), 0, s>>>(cur, H->f32[l], H->cof32[l], nullptr,
@@ -2084,7 +2086,7 @@ cudaError_t mixed_finish(recon_handle *H, double *phi, bool converged)
     if (H->cfg.mixed_df_residual) {
         note_launch(2);
         k_df_sum<<<red_blocks(n), kThreads, 0, s>>>(H->t32[0], H->lo32, n, H->partials,
-                                                    Finish{H->ticket, (double)n, H->scal + S_MEAN_T});
+                                                    Finish{H->ticket, (double)n, H->scal + S_MEAN_T, red_blocks(n)});
         k_df_to_double_gauged<<<stride_blocks(n), kThreads, 0, s>>>(H->t32[0], H->lo32, phi, n,
                                                                    H->scal + S_MEAN_T);
     } else if (converged) {
