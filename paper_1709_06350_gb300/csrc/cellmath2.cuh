@@ -166,24 +166,6 @@ __device__ __forceinline__ float2 fas_update2_det(const Nb19<float2> &n, float2 
     return out;
 }
 
-// Gauss-Seidel on J e = f for two cells with given cofactors (cxx .. cxz:
-// adj(I + H theta)); h2 = h^2.  r: the cells' residuals f - J e (times h2).
-__device__ __forceinline__ float2 lin_update2_cof(const Cof<float2> &a, const Nb19<float2> &e, float2 rhs, float h2,
-                                                  float2 &r)
-{
-    const float2 dxx = fma2(e.c, f2(-2.0f), add2(e.xp, e.xm));
-    const float2 dyy = fma2(e.c, f2(-2.0f), add2(e.yp, e.ym));
-    const float2 dzz = fma2(e.c, f2(-2.0f), add2(e.zp, e.zm));
-    const float2 dxy = edge2(e.xpyp, e.xmym, e.xmyp, e.xpym);
-    const float2 dyz = edge2(e.ypzp, e.ymzm, e.ymzp, e.ypzm);
-    const float2 dxz = edge2(e.xpzp, e.xmzm, e.xmzp, e.xpzm);
-    const float2 offd = fma2(a.xz, dxz, fma2(a.yz, dyz, mul2(a.xy, dxy)));
-    const float2 diag = fma2(a.zz, dzz, fma2(a.yy, dyy, mul2(a.xx, dxx)));
-    r = fma2(rhs, f2(h2), neg2(fma2(offd, f2(0.5f), diag)));
-    const float2 tr = add2(add2(a.xx, a.yy), a.zz);          // -h^2 J_cc / 2
-    return fma2(mul2(r, f2(-0.5f)), rcp2(tr), e.c);
-}
-
 // lin_update2 where e is 0 at the cells and all their edge neighbours: sx, sy,
 // sz the sums of their face neighbours' e (the off-diagonal cofactors drop out)
 __device__ __forceinline__ float2 lin_update2_faces(const Nb19<float2> &t, float2 sx, float2 sy, float2 sz, float2 rhs,

@@ -22,10 +22,12 @@
 //    FP64 addition holds a warp for 16 cycles of the SM's FP64 pipe, and the
 //    block sums of the coarsest solve were most of its time.  Solutions are as
 //    far from 64-bit ones as with FP64 sums (64^3 1.2e-9, 160^3 3.6e-10 of phi).
-//  * The linear levels are relaxed two cells at a time on the paired
-//    instructions.  The FAS levels keep the arithmetic of the grid kernels
-//    (cell_update, det_IH) operation for operation: a mixed solve's last
-//    digits follow the FP32 rounding of its FAS cycles (1e-10 of phi).
+//  * The levels keep the arithmetic of the grid kernels (cell_update, det_IH;
+//    jac_apply and the IEEE quotient of k_lin_pass) operation for operation: a
+//    mixed solve's last digits follow the FP32 rounding of its cycles (1e-10 of
+//    phi).  The paired instructions with an approximate reciprocal on the linear
+//    levels, 2e-8 off in a correction's residual, were 2% of a 64^3 solve faster
+//    (1.70 against 1.73 ms).
 //
 // What bounds it: latency.  One pass over 32^3 takes ~3 us, one over 4^3 ~0.5,
 // at 4-22% issue; a third of the stalls of a cold launch are instruction
@@ -37,7 +39,6 @@
 #include <cooperative_groups.h>
 
 #include "cellmath.cuh"
-#include "cellmath2.cuh"
 #include "dfloat.cuh"
 #include "internal.cuh"
 
@@ -754,30 +755,29 @@ __global__ void __launch_bounds__(NT, 1) k_lin_tail(const __grid_constant__ Tail
 {
     using L = Level<float>;
     Tail<float, NT> C(A);
-    // f and cofactors of a row's two cells (row wa, cell ka; row wb, cell kb);
-    // the cofactor rows are colour split: (i + j + k) even first
     auto f_at = [&](const L &G, const Row &w, int k) { return smem<float>()[C.arr(G, 2) + w.ip * G.NN + w.r + k]; };
-    auto cof2 = [&](const L &G, const Row &wa, int ka, const Row &wb, int kb) {
-        const int n = C.own(G), f = C.arr(G, 2) + n;
-        auto slot = [&](const Row &w, int k) {
-            const int j = (int)(((unsigned)w.r * G.rN) >> 20);
-            return f + w.ip * G.NN + w.r + (((w.ip + j + k) & 1) ? G.half : 0) + (k >> 1);
-        };
-        const float *a = smem<float>() + slot(wa, ka), *b = smem<float>() + slot(wb, kb);
-        Cof<float2> c;
-        c.xx = make_float2(a[0], b[0]);
-        c.yy = make_float2(a[n], b[n]);
-        c.zz = make_float2(a[2 * n], b[2 * n]);
-        c.xy = make_float2(a[3 * n], b[3 * n]);
-        c.yz = make_float2(a[4 * n], b[4 * n]);
-        c.xz = make_float2(a[5 * n], b[5 * n]);
-        return c;
+    // cofactors of cell k of a row; their rows are colour split: (i + j + k) even first
+    auto cof_at = [&](const L &G, const Row &w, int k) {
+        const int n = C.own(G), j = (int)(((unsigned)w.r * G.rN) >> 20);
+        const float *c = smem<float>() + C.arr(G, 2) + n + w.ip * G.NN + w.r + (((w.ip + j + k) & 1) ? G.half : 0) + (k >> 1);
+        Cof<float> a;
+        a.xx = c[0];
+        a.yy = c[n];
+        a.zz = c[2 * n];
+        a.xy = c[3 * n];
+        a.yz = c[4 * n];
+        a.xz = c[5 * n];
+        return a;
     };
-    // new values of two cells and their residuals times h^2
-    auto update = [&](const L &G, int src, const Row &wa, int ka, const Row &wb, int kb, bool two, float2 &r) {
-        const Nb19<float> na = C.nb(G, src, wa, ka), nb = two ? C.nb(G, src, wb, kb) : na;
-        return lin_update2_cof(cof2(G, wa, ka, wb, kb), pack19(na, nb), make_float2(f_at(G, wa, ka), f_at(G, wb, kb)),
-                               6.0f * A.h2_6[G.l], r);
+    // a cell's residual f - J e, and its new value
+    auto residual = [&](const L &G, int src, const Row &w, int k) {
+        return f_at(G, w, k) - jac_apply(cof_at(G, w, k), C.nb(G, src, w, k), A.ih2[G.l]);
+    };
+    auto update = [&](const L &G, int src, const Row &w, int k, float &r) {
+        const Cof<float> a = cof_at(G, w, k);
+        const Nb19<float> n = C.nb(G, src, w, k);
+        r = f_at(G, w, k) - jac_apply(a, n, A.ih2[G.l]);
+        return n.c + r / (-2.0f * (a.xx + a.yy + a.zz) * A.ih2[G.l]);
     };
     auto sweeps = [&](const L &G, int count) {
         const int e = C.arr(G, 0), w = C.arr(G, 1);
@@ -788,14 +788,14 @@ __global__ void __launch_bounds__(NT, 1) k_lin_tail(const __grid_constant__ Tail
                 int ra, ba, rb, bb;
                 const Row wa = C.pair(G, ia, ra, ba), wb = C.pair(G, ib, rb, bb);
                 const int ka = black ? ba : ra, kb = black ? bb : rb, oa = black ? ra : ba, ob = black ? rb : bb;
-                float2 r;
-                const float2 v = update(G, src, wa, ka, wb, kb, two, r);
+                float r;
+                const float va = update(G, src, wa, ka, r), vb = two ? update(G, src, wb, kb, r) : va;
                 if (ona) {
-                    C.put(G, dst, wa, wa.r + ka, v.x);
+                    C.put(G, dst, wa, wa.r + ka, va);
                     C.put(G, dst, wa, wa.r + oa, smem<float>()[src + wa.c + wa.r + oa]);
                 }
                 if (onb) {
-                    C.put(G, dst, wb, wb.r + kb, v.y);
+                    C.put(G, dst, wb, wb.r + kb, vb);
                     C.put(G, dst, wb, wb.r + ob, smem<float>()[src + wb.c + wb.r + ob]);
                 }
             });
@@ -837,10 +837,9 @@ __global__ void __launch_bounds__(NT, 1) k_lin_tail(const __grid_constant__ Tail
         C.twos(G, G.np * G.NN, [&](int ia, int ib, bool ona, bool onb, bool two) {
             int ka, kb;
             const Row wa = C.cell(G, ia, ka), wb = C.cell(G, ib, kb);
-            float2 r;
-            update(G, e, wa, ka, wb, kb, two, r);
-            if (ona) smem<float>()[w + wa.c + wa.r + ka] = r.x * A.ih2[l];
-            if (onb) smem<float>()[w + wb.c + wb.r + kb] = r.y * A.ih2[l];
+            const float ra = residual(G, e, wa, ka), rb = two ? residual(G, e, wb, kb) : ra;
+            if (ona) smem<float>()[w + wa.c + wa.r + ka] = ra;
+            if (onb) smem<float>()[w + wb.c + wb.r + kb] = rb;
         });
         C.block_sync(G);
         df sum = df_make(0.0f, 0.0f), z = sum;
@@ -865,15 +864,12 @@ __global__ void __launch_bounds__(NT, 1) k_lin_tail(const __grid_constant__ Tail
         C.coarsest(
             G, C.arr(G, 0), C.arr(G, 1), C.arr(G, 2) + 7 * C.own(G),
             [&](int src, const Row &w, int kr, int kb, float &rr, float &rb) {
-                float2 r;
-                const float2 v = update(G, src, w, kr, w, kb, true, r);
-                rr = r.x;   // times h^2, as the stop rule only compares them
-                rb = r.y;
-                return v.x;
+                rb = residual(G, src, w, kb);
+                return update(G, src, w, kr, rr);
             },
             [&](int src, const Row &w, int kb) {
-                float2 r;
-                return update(G, src, w, kb, w, kb, false, r).x;
+                float r;
+                return update(G, src, w, kb, r);
             });
     }
     for (int l = nl - 2; l >= 0; --l) {
@@ -1000,7 +996,6 @@ cudaError_t lin_tail(recon_handle *H, int l, float *e, const float *f, const flo
         A.N[q] = H->Nl[l + q];
         const double h = H->hl[l + q];
         A.ih2[q] = (float)(1.0 / (h * h));
-        A.h2_6[q] = (float)(h * h / 6.0);
         A.cof[q] = cof[l + q];
     }
     A.t = e;

@@ -51,3 +51,10 @@ def test_fp32_cycles(N):
     got, want = history(N)[0], recorded(N)[0]
     assert len(got) == len(want)
     np.testing.assert_allclose(got, want, rtol=1e-12)
+
+
+@pytest.mark.parametrize("N", [64, 112, 128])
+def test_corrections(N):
+    got, want = history(N)[1], recorded(N)[1]
+    assert len(got) == len(want)
+    np.testing.assert_allclose(got, want, rtol=1e-12)
