@@ -17,7 +17,7 @@
 //
 // The quantile is FP64 and was half of the time (normcdfinv, ~67 FP64
 // operations per value at one per 64 FP32 ones): it is evaluated once per 128
-// ranks and continued by its Taylor series (four FP64 operations per value).
+// ranks and continued by its Taylor series (five FP64 operations per value).
 // What bounds it: the sector traffic of the scatters and the FP64 pipe.
 // Measured (GB300): 256^3 4.24 -> 1.35 to 1.49 ms (GPUs differ), 512^3
 // 36.9 -> 12.1 ms; a 256^3 field of rounded values (radix path) 4.2 -> 2.9 ms.
@@ -248,33 +248,32 @@ k_gauss_scatter(const double *__restrict__ v, size_t n, const GaussPlan *__restr
 // to r is P_k(z) D^k, P_1 = 1, P_{k+1} = P_k' + k z P_k; the series about the
 // middle of 128 ranks in terms of their offset is kept per anchor.  From rank
 // kTail on an offset is below 2^-8 of the rank and six terms leave 2^-58; the
-// terms from the fourth on are below 2^-32 and evaluated in FP32.  The lower
-// half is mirrored, so the two tails have the same precision.
+// terms from the fourth on are below 2^-32 and evaluated in FP32, for z itself:
+// with std in them they left FP32's range (infinities from std 3e56 up, 2e-11
+// of std lost below 1e-24).  The lower half is mirrored, so the two tails have
+// the same precision.
 constexpr int kAnchor = 128;
 constexpr size_t kTail = 16384;
 struct __align__(64) Anchor {
-    double below, above;                     // mean + sd z, mean - sd z
-    double c1, c2, c3;
-    float c4, c5, c6, unused;
+    double z, c1, c2, c3;
+    float c4, c5, c6, unused[5];
 };
 __global__ void __launch_bounds__(kThreads)
-k_gauss_anchors(size_t n, size_t count, const GaussPlan *__restrict__ P, Anchor *__restrict__ out)
+k_gauss_anchors(size_t n, size_t count, Anchor *__restrict__ out)
 {
     const size_t a = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (a >= count) return;
-    const double z = normcdfinv(((double)(a * kAnchor + kAnchor / 2) + 0.5) / (double)n), z2 = z * z, sd = P->sd;
+    const double z = normcdfinv(((double)(a * kAnchor + kAnchor / 2) + 0.5) / (double)n), z2 = z * z;
     const double D = 2.5066282746310002 * exp(0.5 * z2) / (double)n;   // sqrt(2 pi)
     const double D2 = D * D, D3 = D2 * D;
     Anchor x;
-    x.below = P->mean + sd * z;
-    x.above = P->mean - sd * z;
-    x.c1 = sd * D;
-    x.c2 = sd * D2 * z * 0.5;
-    x.c3 = sd * D3 * (1.0 + 2.0 * z2) * (1.0 / 6.0);
-    x.c4 = (float)(sd * D2 * D2 * z * (7.0 + 6.0 * z2) * (1.0 / 24.0));
-    x.c5 = (float)(sd * D2 * D3 * (7.0 + z2 * (46.0 + 24.0 * z2)) * (1.0 / 120.0));
-    x.c6 = (float)(sd * D3 * D3 * z * (127.0 + z2 * (326.0 + 120.0 * z2)) * (1.0 / 720.0));
-    x.unused = 0.0f;
+    x.z = z;
+    x.c1 = D;
+    x.c2 = D2 * z * 0.5;
+    x.c3 = D3 * (1.0 + 2.0 * z2) * (1.0 / 6.0);
+    x.c4 = (float)(D2 * D2 * z * (7.0 + 6.0 * z2) * (1.0 / 24.0));
+    x.c5 = (float)(D2 * D3 * (7.0 + z2 * (46.0 + 24.0 * z2)) * (1.0 / 120.0));
+    x.c6 = (float)(D3 * D3 * z * (127.0 + z2 * (326.0 + 120.0 * z2)) * (1.0 / 720.0));
     out[a] = x;
 }
 __device__ __noinline__ double quantile_tail(size_t lo, bool low, size_t n, double m, double sd)
@@ -290,8 +289,8 @@ __device__ __forceinline__ double quantile(size_t r, size_t n, const GaussPlan *
     const float f = (float)((int)(lo & (kAnchor - 1)) - kAnchor / 2);
     const double d = df_f2d_bits(f);
     const double p = df_f2d_bits(fmaf(fmaf(x.c6, f, x.c5), f, x.c4));
-    const double t = fma(fma(fma(p, d, x.c3), d, x.c2), d, x.c1);
-    return r == lo ? fma(t, d, x.below) : fma(-t, d, x.above);
+    const double z = fma(fma(fma(fma(p, d, x.c3), d, x.c2), d, x.c1), d, x.z);
+    return fma(r == lo ? P->sd : -P->sd, z, P->mean);
 }
 
 // rank of every member within its bucket, and its quantile to its place
@@ -539,7 +538,7 @@ cudaError_t gaussianise(recon_handle *H, const double *v, size_t n, double *g)
     note_launch(5);
     k_gauss_stats<<<nb, kThreads, 0, s>>>(v, n, H->partials);
     k_gauss_moments<<<1, kReduceThreads, 0, s>>>(H->partials, (int)nb, (double)n, P);
-    k_gauss_anchors<<<blocks_for(nanchor), kThreads, 0, s>>>(n, nanchor, P, anchors);
+    k_gauss_anchors<<<blocks_for(nanchor), kThreads, 0, s>>>(n, nanchor, anchors);
     k_gauss_sample<<<(unsigned)(sblocks < 608 ? sblocks : 608), kSampleRun, 0, s>>>(v, n, step, P);
     k_gauss_plan<<<1, kScanThreads, 0, s>>>(whole ? 1 : kSampleStep / kSampleRun, P);
     // buckets
