@@ -200,11 +200,13 @@ __device__ __forceinline__ float cell_update(const Nb19<float> &n, float rhs, fl
     return n.c - h2_6 * (sn - s);
 }
 
-// a / b for positive normal b, within 1 ulp (Newton's iteration for 1 / b, with
-// Markstein's remainder step for the quotient): the hardware's reciprocal
-// approximation, one Newton step on 1 / b (to ~40 bits) and one on the
-// quotient, whose remainder is exact in one fma.  Four FP64 operations and no
-// branch; FP64 operations are what the FP64 smoother waits for.
+// a / b within 1 ulp, where b is positive and b, 1 / b and the quotient are
+// normal numbers (b from 2^-1022 to 2^1022; beyond, the reciprocal is flushed
+// to zero or infinity).  Newton's iteration for 1 / b, with Markstein's
+// remainder step for the quotient: the hardware's reciprocal approximation, one
+// Newton step on 1 / b (to ~40 bits) and one on the quotient, whose remainder
+// is exact in one fma.  Four FP64 operations and no branch; FP64 operations are
+// what the FP64 smoother waits for.
 __device__ __forceinline__ double div_pos(double a, double b)
 {
     double r;
