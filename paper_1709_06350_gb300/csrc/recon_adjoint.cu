@@ -313,7 +313,7 @@ k_jt_fine(const T *__restrict__ phi, const T *__restrict__ lam, const T *__restr
             if (MODE == 0) {
                 const T l0 = lc[o];
                 if (((p + j + k) & 1) == colour) {
-                    const T diag = -2.0 * (cc[o] + cc[kFCP + o] + cc[2 * kFCP + o]) * ih2;
+                    const T diag = T(-2) * (cc[o] + cc[kFCP + o] + cc[2 * kFCP + o]) * ih2;
                     out[id] = l0 + (f[id] - jt_here()) / diag;
                 } else {
                     out[id] = l0;
