@@ -285,9 +285,10 @@ recon_status recon_gaussianise(recon_handle *h, const double *field, double *out
  *   J^T lam + mu 1 = gbar_phi,  sum(lam) = 0,  J = d det(I + H phi)/d phi.
  * lam and the residual of this equation are FP64, to a relative residual of
  * 1e-12; on grids above 32^3 the corrections between two residuals are FP32
- * multigrid cycles (FP64 ones where those do not get there).
- * Errors: RECON_E_INVALID (no previous solve), RECON_E_NOCONV,
- * RECON_E_CUDA, RECON_E_UNIMPLEMENTED (not available in this build). */
+ * multigrid cycles (FP64 ones where those do not get there, or where their
+ * arrays do not fit in device memory beside the FP64 ones).
+ * Errors: RECON_E_INVALID (no previous solve), RECON_E_NOCONV (a relative
+ * residual of 1e-8 not reached), RECON_E_OOM, RECON_E_CUDA, RECON_E_UNIMPLEMENTED (not available in this build). */
 recon_status recon_adjoint(recon_handle *h, const double *gbar_phi, double *gbar_b);
 
 /* ---------------------------------------------------------------------------

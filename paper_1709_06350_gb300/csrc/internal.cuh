@@ -28,7 +28,7 @@ struct AdjWork {
     double null_rel = 0.0;
     double *th[kMaxLevels] = {}, *cof[kMaxLevels] = {}, *lam[kMaxLevels] = {}, *f[kMaxLevels] = {};
     double *nvec = nullptr;
-    // FP32 corrections: levels 1.. (cof32[0] if stored0)
+    bool mixed = false;        // the FP32 corrections' arrays are held: levels 1.. (cof32[0] if stored0)
     float *cof32[kMaxLevels] = {}, *lam32[kMaxLevels] = {}, *f32[kMaxLevels] = {};
     bool cof32_ready = false, cof64_ready = false;   // cofactors match the last solve
     bool ready64 = false;      // the FP64 coarse levels are allocated

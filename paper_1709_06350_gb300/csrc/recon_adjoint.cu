@@ -729,6 +729,33 @@ cudaError_t fine_attr()
     return cudaFuncSetAttribute(k_jt_fine<2, T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)fine_smem<T>());
 }
 
+// the arrays of the FP32 corrections
+void free32(AdjWork &A)
+{
+    for (int l = 0; l < kMaxLevels; ++l)
+        for (float **p : {&A.lam32[l], &A.f32[l], &A.cof32[l]}) {
+            if (*p) cudaFree(*p);
+            *p = nullptr;
+        }
+    A.mixed = A.cof32_ready = false;
+}
+cudaError_t alloc32(recon_handle *H)
+{
+    AdjWork &A = H->adj;
+    for (int l = 0; l < H->nlev; ++l) {
+        const size_t n = ncell(H->Nl[l]);
+        if (l > 0) {
+            CK(cudaMalloc(&A.lam32[l], sizeof(float) * n));
+            CK(cudaMalloc(&A.f32[l], sizeof(float) * n));
+        }
+        if (l > 0 || A.stored0) CK(cudaMalloc(&A.cof32[l], sizeof(float) * 6 * n));
+    }
+    return cudaSuccess;
+}
+
+// The FP32 corrections' arrays come last: where they do not fit, the solves run
+// in FP64 throughout, and where its coarse levels do not fit beside them, they
+// make room.  A grid needs no more memory than FP64 alone needs.
 cudaError_t adj_alloc(recon_handle *H)
 {
     AdjWork &A = H->adj;
@@ -737,17 +764,18 @@ cudaError_t adj_alloc(recon_handle *H)
     CK(fine_attr<double>());
     CK(fine_attr<float>());
     if (A.stored0) CK(cudaMalloc(&A.cof[0], sizeof(double) * 6 * ncell(H->N)));
-    if (mixed_ok(H))
-        for (int l = 0; l < H->nlev; ++l) {
-            const size_t n = ncell(H->Nl[l]);
-            if (l > 0) {
-                CK(cudaMalloc(&A.lam32[l], sizeof(float) * n));
-                CK(cudaMalloc(&A.f32[l], sizeof(float) * n));
-            }
-            if (l > 0 || A.stored0) CK(cudaMalloc(&A.cof32[l], sizeof(float) * 6 * n));
-        }
     CK(cudaMalloc(&A.nvec, sizeof(double) * ncell(H->N)));
     CK(cudaMalloc(&A.f[0], sizeof(double) * ncell(H->N)));
+    A.mixed = mixed_ok(H);
+    if (A.mixed) {
+        const cudaError_t e = alloc32(H);
+        if (e == cudaErrorMemoryAllocation) {
+            cudaGetLastError();
+            free32(A);
+        } else if (e != cudaSuccess) {
+            return e;
+        }
+    }
     A.ready = true;
     return cudaSuccess;
 }
@@ -773,7 +801,13 @@ cudaError_t setup64(recon_handle *H)
 {
     AdjWork &A = H->adj;
     if (A.cof64_ready) return cudaSuccess;
-    CK(alloc64(H));
+    cudaError_t e = alloc64(H);
+    if (e == cudaErrorMemoryAllocation && A.mixed) {   // in place of the FP32 corrections' arrays
+        cudaGetLastError();
+        free32(A);
+        e = alloc64(H);
+    }
+    CK(e);
     for (int l = 1; l < H->nlev; ++l) {
         CK(restrict_plain<double>(H->Nl[l - 1], l > 1 ? A.th[l - 1] : H->last_phi, A.th[l], H->stream));
         note_launch();
@@ -824,29 +858,28 @@ cudaError_t setup_mixed(recon_handle *H, const JtHier<float> &Y)
 }
 
 // J^T lam = f from lam = 0: mixed, and in FP64 from where that ends if it
-// stops short of tol (or the grid is too small for it)
+// stops short of tol (or the grid is too small for it).  The V-cycles taken, or
+// one of the two errors.
+constexpr int kFailed = -1, kNoMemory = -2;
 int solve_jt(recon_handle *H, double *lam, const double *f, double tol, int max_cycles, double *rel)
 {
     int c = 0;
     *rel = 1.0;
-    if (mixed_ok(H)) {
+    if (H->adj.mixed) {
         const JtHier<float> Y = hier_mixed(H);
         const size_t n = ncell(H->N);
         note_launch();
         k_narrow<<<stride_blocks(n), kThreads, 0, H->stream>>>(H->last_phi, Y.th[0], n);
         if (!H->adj.cof32_ready) {
-            if (setup_mixed(H, Y) != cudaSuccess) return -1;
+            if (setup_mixed(H, Y) != cudaSuccess) return kFailed;
             H->adj.cof32_ready = true;
         }
         c = jt_solve_mixed(H, Y, lam, f, tol, max_cycles, rel);
         if (c < 0 || *rel < tol || c >= max_cycles) return c;
     }
     const bool zero = c == 0 || !std::isfinite(*rel) || *rel > 1.0;   // (a diverged correction is dropped)
-    if (setup64(H) != cudaSuccess) {
-        // the FP64 workspace does not fit: keep the mixed answer if there is one
-        cudaGetLastError();
-        return zero ? -1 : c;
-    }
+    const cudaError_t e = setup64(H);
+    if (e != cudaSuccess) return e == cudaErrorMemoryAllocation ? kNoMemory : kFailed;
     const int d = jt_solve(H, lam, f, tol, max_cycles - c, zero, rel);
     return d < 0 ? d : c + d;
 }
@@ -863,12 +896,22 @@ void adj_free(recon_handle *H)
         }
         if (A.f[l]) cudaFree(A.f[l]);
         if (A.cof[l]) cudaFree(A.cof[l]);
-        if (A.lam32[l]) cudaFree(A.lam32[l]);
-        if (A.f32[l]) cudaFree(A.f32[l]);
-        if (A.cof32[l]) cudaFree(A.cof32[l]);
     }
+    free32(A);
     if (A.nvec) cudaFree(A.nvec);
     A = AdjWork{};
+}
+
+static recon_status failed(recon_handle *H, int code, const char *what)
+{
+    if (code != kNoMemory) {
+        H->err = what;
+        return RECON_E_CUDA;
+    }
+    adj_free(H);
+    cudaGetLastError();
+    H->err = "adjoint workspace allocation failed";
+    return RECON_E_OOM;
 }
 
 recon_status adjoint(recon_handle *H, const double *gbar, double *lam)
@@ -914,10 +957,7 @@ recon_status adjoint(recon_handle *H, const double *gbar, double *lam)
                 H->last_phi, nullptr, nullptr, A.f[0], N, 1.0 / (H->h * H->h), 0, -1.0, H->partials, nullptr, 1.0);
         double rel = 0.0;
         const int c1 = solve_jt(H, A.nvec, A.f[0], tol, maxc, &rel);
-        if (c1 < 0) {
-            H->err = "adjoint null-vector solve failed";
-            return RECON_E_CUDA;
-        }
+        if (c1 < 0) return failed(H, c1, "adjoint null-vector solve failed");
         note_launch();
         k_add_one<<<blocks_for(n), kThreads, 0, s>>>(A.nvec, n);
         A.null_ready = true;
@@ -932,10 +972,7 @@ recon_status adjoint(recon_handle *H, const double *gbar, double *lam)
     k_sub_mean<double><<<blocks_for(n), kThreads, 0, s>>>(A.f[0], n, H->scal + S_ADJ_MEAN);
     double rel = 0.0;
     const int c2 = solve_jt(H, lam, A.f[0], tol, maxc, &rel);
-    if (c2 < 0) {
-        H->err = "adjoint solve failed";
-        return RECON_E_CUDA;
-    }
+    if (c2 < 0) return failed(H, c2, "adjoint solve failed");
     // lam -= (sum lam / sum n) n
     note_launch(5);
     k_sum<<<nred(n), kThreads, 0, s>>>(lam, n, H->partials);
