@@ -163,8 +163,8 @@ __device__ __forceinline__ double block_min(double v, double *sh)
 }
 
 // True in every thread of the block of the grid that finishes last (each
-// block calls it after thread 0 stored the block's partial results, which the
-// last block may then read); the counter is left at 0 for the next kernel.
+// block calls it after thread 0 stored the block's partial results, or any
+// thread before a barrier, and the last block may then read them); the counter is left at 0 for the next kernel.
 // Finishing a grid-wide sum in its own kernel instead of a one-block launch
 // behind it saves that launch: 5-10 us each, a tenth of a 64^3 solve.
 __device__ __forceinline__ bool last_block(unsigned *counter)
@@ -194,6 +194,8 @@ inline unsigned row_groups(int N) { return row_grid(N, kMaxRedBlocks); }
 // restriction: 461 us with 2048 blocks, two per SM, about 400 us with one wave)
 constexpr unsigned kSMs = 152;
 inline unsigned wave_grid(int N, unsigned per_sm) { return row_grid(N, kSMs * per_sm); }
+constexpr int kMaxTurns = 7;   // groups that a block takes at most, from two blocks per SM on
+static_assert(kMaxTurns * 2 * kSMs >= kMaxRedBlocks, "");
 
 // Totals of columns 0 .. K-1 of the groups' partials (4 doubles each) in a
 // fixed order, that of a block of kReduceThreads, in ltid() == 0 of a block of
@@ -213,12 +215,15 @@ __device__ __forceinline__ void total_columns(const double *partials, int nb, do
         }
     __syncthreads();
 #pragma unroll
-    for (int u = 0; u < kRounds; ++u)
+    for (int u = 0; u < kRounds; ++u) {
+        const int first = u * NT + (ltid() & ~31);
         for (int x = 0; x < K; ++x) {
             double v = p[u][0][x] + p[u][1][x];
-            for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-            if ((ltid() & 31) == 0) sh[x * kWarps + (u * NT + ltid()) / 32] = v;
+            if (first < nb)   // (else 32 zeros)
+                for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+            if ((ltid() & 31) == 0) sh[x * kWarps + first / 32] = v;
         }
+    }
     __syncthreads();
     for (int x = 0; x < K; ++x) {
         out[x] = 0.0;

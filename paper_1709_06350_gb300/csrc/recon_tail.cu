@@ -25,9 +25,9 @@
 //  * The levels keep the arithmetic of the grid kernels (cell_update, det_IH;
 //    jac_apply and the IEEE quotient of k_lin_pass) operation for operation: a
 //    mixed solve's last digits follow the FP32 rounding of its cycles (1e-10 of
-//    phi).  The paired instructions with an approximate reciprocal on the linear
-//    levels, 2e-8 off in a correction's residual, were 2% of a 64^3 solve faster
-//    (1.70 against 1.73 ms).
+//    phi).  Paired instructions with an approximate reciprocal on the linear
+//    levels, 2e-8 off in a correction's residual, were no faster (64^3 solve
+//    1.68 ms either way; linear tail of 160^3 194 against 197 us).
 //
 // What bounds it: latency.  One pass over 32^3 takes ~3 us, one over 4^3 ~0.5,
 // at 4-22% issue; a third of the stalls of a cold launch are instruction
