@@ -288,7 +288,8 @@ recon_status recon_gaussianise(recon_handle *h, const double *field, double *out
  * multigrid cycles (FP64 ones where those do not get there, or where their
  * arrays do not fit in device memory beside the FP64 ones).
  * Errors: RECON_E_INVALID (no previous solve), RECON_E_NOCONV (a relative
- * residual of 1e-8 not reached), RECON_E_OOM, RECON_E_CUDA, RECON_E_UNIMPLEMENTED (not available in this build). */
+ * residual of 1e-8 not reached), RECON_E_OOM, RECON_E_CUDA,
+ * RECON_E_UNIMPLEMENTED (not available in this build). */
 recon_status recon_adjoint(recon_handle *h, const double *gbar_phi, double *gbar_b);
 
 /* ---------------------------------------------------------------------------

@@ -10,10 +10,7 @@ constexpr int kMaxLevels = 16;
 using recon::kMaxRedBlocks;
 constexpr int kFusedMinN = 128;       // grids of at least this size use the fused sweeps
 
-// Workspace of the adjoint (allocated at its first call): the potential of
-// every coarse level, the six cofactor arrays of every level, the iterate and
-// right side of every coarse level, the null vector of J^T.
-// workspace of recon_gaussianise (allocated at its first call)
+// Workspace of recon_gaussianise (allocated at its first call)
 struct GaussWork {
     size_t cap = 0;
     void *pairs = nullptr;      // 24 bytes per value: (key, index) pairs or bucket members
@@ -21,6 +18,9 @@ struct GaussWork {
     void *anchors = nullptr, *plan = nullptr;
 };
 
+// Workspace of the adjoint (allocated at its first call): the potential of
+// every coarse level, the six cofactor arrays of every level, the iterate and
+// right side of every coarse level, the null vector of J^T.
 struct AdjWork {
     bool ready = false;
     bool stored0 = true;       // the finest level's cofactors are kept (else formed in every J^T)

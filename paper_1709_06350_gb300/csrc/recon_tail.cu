@@ -20,8 +20,9 @@
 //    barriers; if it was the last, the extra red pass is dropped.
 //  * Sums are double-float (48 bits) for FP32 levels, FP64 for FP64 ones: an
 //    FP64 addition holds a warp for 16 cycles of the SM's FP64 pipe, and the
-//    block sums of the coarsest solve were most of its time.  Solutions are as
-//    far from 64-bit ones as with FP64 sums (64^3 1.2e-9, 160^3 3.6e-10 of phi).
+//    block sums of the coarsest solve were most of its time.  The cycles of
+//    mixed solves are bit for bit those with FP64 sums and a two-pass variance
+//    (12 boxes, 64^3 to 448^3).
 //  * The levels keep the arithmetic of the grid kernels (cell_update, det_IH;
 //    jac_apply and the IEEE quotient of k_lin_pass) operation for operation: a
 //    mixed solve's last digits follow the FP32 rounding of its cycles (1e-10 of
@@ -29,9 +30,10 @@
 //    levels, 2e-8 off in a correction's residual, were no faster (64^3 solve
 //    1.68 ms either way; linear tail of 160^3 194 against 197 us).
 //
-// What bounds it: latency.  One pass over 32^3 takes ~3 us, one over 4^3 ~0.5,
-// at 4-22% issue; a third of the stalls of a cold launch are instruction
-// fetches.  16 blocks instead of 8 measured the same (32^3: 91 against 93 us
+// What bounds it: latency.  One pass over 32^3 takes ~3 us, one over 4^3 ~0.5;
+// issue is active 11-12% of the time (160^3's tails, 20^3 and 10^3), and most
+// stalls are at barriers, of the blocks and warps that wait for block 0's small
+// levels.  16 blocks instead of 8 measured the same (32^3: 91 against 93 us
 // per cycle) and a batch of solves slower.  Measured (GB300), against one
 // thread block from 16^3 down and a dozen launches per level above it: mixed
 // solves at 64^3 2.83 -> 1.77 ms, 160^3 (ends at 10^3) 8.78 -> 5.92 ms, FP64
@@ -917,9 +919,14 @@ size_t place(TailArgs<T> &A, bool lin)
     return c * sizeof(T);
 }
 
+// dynamic shared memory: the linear tail of 32^3 and below takes 207360 bytes,
+// the most of any side; the static part stays below 6 KB
+constexpr int kTailSmem = 208 * 1024;
+
 template <typename T>
 cudaError_t launch(void (*kern)(TailArgs<T>), const TailArgs<T> &A, size_t smem, int threads, cudaStream_t s)
 {
+    if (smem > (size_t)kTailSmem) return cudaErrorInvalidValue;
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute at[1];
     const unsigned n = A.dist ? kTailCtas : 1;
@@ -936,14 +943,10 @@ cudaError_t launch(void (*kern)(TailArgs<T>), const TailArgs<T> &A, size_t smem,
     return cudaLaunchKernelEx(&cfg, kern, A);
 }
 
-// dynamic shared memory: the linear tail of 32^3 and below takes 204 KB; the
-// static part stays below 6 KB
-constexpr int kTailSmem = 208 * 1024;
-
 }  // namespace
 
 // A level starts a tail when it has at most this many cells: 32^3 for FP32
-// (the linear tail's arrays of 32^3 and below fill 209 KB in each block);
+// (the linear tail's arrays of 32^3 and below fill each block's memory);
 // 16^3 for FP64, whose larger levels need more SMs for their FP64 rate.
 template <typename T>
 bool tail_ok(int N)
