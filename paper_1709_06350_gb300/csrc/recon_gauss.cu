@@ -21,8 +21,10 @@
 // What bounds it: the sector traffic of the scatters and the FP64 pipe.
 // Measured (GB300): 256^3 4.24 -> 1.35 to 1.49 ms (GPUs differ; scatter 0.43,
 // ranks 0.38, places 0.16), 512^3 36.9 -> 12.1 to 12.7 ms; a 256^3 field of
-// rounded values (radix path) 4.2 -> 2.9 ms.
+// rounded values (radix path) 3.5 -> 1.8 ms.  Fields that take the radix path are
+// 3 to 5% slower than by it alone at 64^3 and 80^3, and faster at other sides.
 #include <climits>
+#include <cmath>
 
 #include "dfloat.cuh"
 #include "internal.cuh"
@@ -77,9 +79,56 @@ __device__ __forceinline__ unsigned long long linear_bits(const GaussPlan *P, do
     return u < 0 ? 0ull : (u >= (1ll << 52) ? (1ull << 52) - 1 : (unsigned long long)u);
 }
 
-// per-block sums of v and v^2, smallest and largest key
+// mean, population std, the linear map; clears the cells (one block of kThreads)
+__device__ __noinline__ void gauss_moments(const double *partials, int nb, double n, GaussPlan *P)
+{
+    __shared__ double sh[2 * 32];
+    __shared__ unsigned long long smin[kThreads / 32], smax[kThreads / 32];
+    double sums[2];
+    total_columns<kThreads>(partials, nb, sh, sums);
+    unsigned long long kmin = ~0ull, kmax = 0ull;
+    for (int i = threadIdx.x; i < nb; i += kThreads) {
+        const unsigned long long x = (unsigned long long)__double_as_longlong(__ldcg(partials + 4 * i + 2));
+        const unsigned long long y = (unsigned long long)__double_as_longlong(__ldcg(partials + 4 * i + 3));
+        kmin = x < kmin ? x : kmin;
+        kmax = y > kmax ? y : kmax;
+    }
+    for (int o = 16; o > 0; o >>= 1) {
+        const unsigned long long x = __shfl_xor_sync(0xffffffffu, kmin, o), y = __shfl_xor_sync(0xffffffffu, kmax, o);
+        kmin = x < kmin ? x : kmin;
+        kmax = y > kmax ? y : kmax;
+    }
+    if ((threadIdx.x & 31) == 0) {
+        smin[threadIdx.x >> 5] = kmin;
+        smax[threadIdx.x >> 5] = kmax;
+    }
+    for (int c = threadIdx.x; c < kCells; c += kThreads) P->cell[c] = 0;
+    __syncthreads();
+    if (ltid() == 0) {
+        for (int w = 1; w < kThreads / 32; ++w) {
+            kmin = smin[w] < kmin ? smin[w] : kmin;
+            kmax = smax[w] > kmax ? smax[w] : kmax;
+        }
+        const double m = sums[0] / n, var = sums[1] / n - m * m;
+        P->mean = m;
+        P->sd = var > 0.0 ? sqrt(var) : 0.0;
+        const double lo = key_value(kmin), range = key_value(kmax) - lo;
+        P->squares = 0;
+        // (equal values, ranges that overflow or underflow the significand map)
+        P->bad = !(range > 1e-290 && range < 1e290 && fabs(lo) < 1e290);
+        int e = 0;
+        frexp(range, &e);                    // range < 2^e
+        const double top = ldexp(1.0, P->bad ? 0 : e);
+        P->shift = top - lo;
+        P->base = (unsigned long long)__double_as_longlong(top);
+    }
+}
+
+// per-block sums of v and v^2, smallest and largest key; the last block makes
+// the moments and the map of them
 __global__ void __launch_bounds__(kThreads)
-k_gauss_stats(const double *__restrict__ v, size_t n, double *__restrict__ partials)
+k_gauss_stats(const double *__restrict__ v, size_t n, double *__restrict__ partials, unsigned *__restrict__ counter,
+              GaussPlan *__restrict__ P)
 {
     __shared__ double sh[32];
     __shared__ unsigned long long smin[kThreads / 32], smax[kThreads / 32];
@@ -114,112 +163,44 @@ k_gauss_stats(const double *__restrict__ v, size_t n, double *__restrict__ parti
         partials[4 * blockIdx.x + 2] = __longlong_as_double((long long)kmin);
         partials[4 * blockIdx.x + 3] = __longlong_as_double((long long)kmax);
     }
-}
-
-// mean, population std, the linear map; clears the cells
-__global__ void __launch_bounds__(kReduceThreads)
-k_gauss_moments(const double *__restrict__ partials, int nb, double n, GaussPlan *__restrict__ P)
-{
-    __shared__ double sh[32];
-    __shared__ unsigned long long smin[32], smax[32];
-    double a = 0.0, b = 0.0;
-    unsigned long long kmin = ~0ull, kmax = 0ull;
-    for (int i = threadIdx.x; i < nb; i += blockDim.x) {
-        a += partials[4 * i + 0];
-        b += partials[4 * i + 1];
-        const unsigned long long x = (unsigned long long)__double_as_longlong(partials[4 * i + 2]);
-        const unsigned long long y = (unsigned long long)__double_as_longlong(partials[4 * i + 3]);
-        kmin = x < kmin ? x : kmin;
-        kmax = y > kmax ? y : kmax;
-    }
-    for (int o = 16; o > 0; o >>= 1) {
-        const unsigned long long x = __shfl_xor_sync(0xffffffffu, kmin, o), y = __shfl_xor_sync(0xffffffffu, kmax, o);
-        kmin = x < kmin ? x : kmin;
-        kmax = y > kmax ? y : kmax;
-    }
-    if ((threadIdx.x & 31) == 0) {
-        smin[threadIdx.x >> 5] = kmin;
-        smax[threadIdx.x >> 5] = kmax;
-    }
-    a = block_sum<kReduceThreads>(a, sh);
-    b = block_sum<kReduceThreads>(b, sh);
-    for (int c = threadIdx.x; c < kCells; c += blockDim.x) P->cell[c] = 0;
-    if (ltid() == 0) {
-        for (int w = 1; w < kReduceThreads / 32; ++w) {
-            kmin = smin[w] < kmin ? smin[w] : kmin;
-            kmax = smax[w] > kmax ? smax[w] : kmax;
-        }
-        const double m = a / n, var = b / n - m * m;
-        P->mean = m;
-        P->sd = var > 0.0 ? sqrt(var) : 0.0;
-        const double lo = key_value(kmin), range = key_value(kmax) - lo;
-        P->squares = 0;
-        // (equal values, ranges that overflow or underflow the significand map)
-        P->bad = !(range > 1e-290 && range < 1e290 && fabs(lo) < 1e290);
-        int e = 0;
-        frexp(range, &e);                    // range < 2^e
-        const double top = ldexp(1.0, P->bad ? 0 : e);
-        P->shift = top - lo;
-        P->base = (unsigned long long)__double_as_longlong(top);
-    }
-}
-
-// cell counts of the sample (kSampleRun of every kSampleStep values, or all of a small field)
-__global__ void __launch_bounds__(kSampleRun)
-k_gauss_sample(const double *__restrict__ v, size_t n, size_t step, GaussPlan *__restrict__ P)
-{
-    __shared__ unsigned c[kCells];
-    if (P->bad) return;
-    for (int i = threadIdx.x; i < kCells; i += kSampleRun) c[i] = 0;
-    __syncthreads();
-    for (size_t b = (size_t)blockIdx.x * step; b < n; b += (size_t)gridDim.x * step)
-        if (b + threadIdx.x < n) atomicAdd(&c[linear_bits(P, v[b + threadIdx.x]) >> kCellBits], 1u);
-    __syncthreads();
-    for (int i = threadIdx.x; i < kCells; i += kSampleRun)
-        if (c[i]) atomicAdd(&P->cell[i], c[i]);
+    if (last_block(counter)) gauss_moments(partials, gridDim.x, (double)n, P);
 }
 
 __device__ __forceinline__ unsigned block_excl_scan(unsigned v, unsigned *sh, unsigned *total);
 
-// sub-buckets of every cell: a power of two above its share / kPerBucket
-// (below n / 8 + kCells buckets in all)
-__global__ void __launch_bounds__(kScanThreads)
-k_gauss_plan(int weight, GaussPlan *__restrict__ P)
-{
-    __shared__ unsigned sh[32];
-    constexpr int kPer = kCells / kScanThreads;
-    unsigned lg[kPer], sum = 0;
-    for (int i = 0; i < kPer; ++i) {
-        const unsigned want = (P->cell[threadIdx.x * kPer + i] * (unsigned)weight) / kPerBucket;
-        lg[i] = want ? 32 - __clz(want) - (__popc(want) == 1) : 0;   // ceil(log2(want))
-        sum += 1u << lg[i];
-    }
-    unsigned total;
-    unsigned run = block_excl_scan(sum, sh, &total);
-    for (int i = 0; i < kPer; ++i) {
-        P->cell[threadIdx.x * kPer + i] = run;
-        P->down[threadIdx.x * kPer + i] = (unsigned char)(kCellBits - lg[i]);
-        run += 1u << lg[i];
-    }
-}
-
-// bucket of every value and its place among the bucket's arrivals
-// (a bucket that alone would take a sixteenth of kMaxWork ends it early: its
-// arrivals queue on one counter)
+// bucket of every value and its place among the bucket's arrivals.  Arrivals at
+// one counter queue (2.3 ns each), so a warp takes the places of one bucket by one
+// atomic, and a bucket that alone would take a sixteenth of kMaxWork (`most`
+// values) ends the count: stored by the arrival that fills it, not by all after it
+// (160^3, half of it zeros: 1.41 ms before the radix sort began).  The flag is read
+// every fourth turn: read every turn, its one cache line took 0.15 ms at 256^3.
 __global__ void __launch_bounds__(kThreads)
 k_gauss_count(const double *__restrict__ v, size_t n, GaussPlan *__restrict__ P, unsigned *__restrict__ counts,
-              uint2 *__restrict__ where)
+              uint2 *__restrict__ where, unsigned most)
 {
     volatile int *bad = &P->bad;
+    const unsigned lane = threadIdx.x & 31;
+    const size_t stride = (size_t)gridDim.x * blockDim.x;
     int turn = 0;
-    for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
-        if ((turn++ & 3) == 0 && *bad) return;
-        const unsigned long long u = linear_bits(P, __ldcs(v + i));
-        const unsigned c = (unsigned)(u >> kCellBits);
-        const unsigned b = P->cell[c] + (unsigned)((u & ((1ull << kCellBits) - 1)) >> P->down[c]);
-        const unsigned long long at = atomicAdd(&counts[b], 1u);
-        __stcs(where + i, make_uint2(b, (unsigned)at));
-        if (at * at > kMaxWork / 16 * n) *bad = 1;
+    for (size_t first = (size_t)blockIdx.x * blockDim.x + (threadIdx.x - lane); first < n; first += stride) {
+        if ((turn++ & 3) == 0 && __any_sync(0xffffffffu, *bad)) return;
+        const size_t i = first + lane;
+        const bool on = i < n;
+        unsigned b = ~0u;
+        if (on) {
+            const unsigned long long u = linear_bits(P, __ldcs(v + i));
+            const unsigned c = (unsigned)(u >> kCellBits);
+            b = P->cell[c] + (unsigned)((u & ((1ull << kCellBits) - 1)) >> P->down[c]);
+        }
+        const unsigned peers = __match_any_sync(0xffffffffu, b);
+        const int leader = __ffs(peers) - 1;
+        unsigned at = 0;
+        if (on && (int)lane == leader) at = atomicAdd(&counts[b], (unsigned)__popc(peers));
+        at = __shfl_sync(0xffffffffu, at, leader) + __popc(peers & ((1u << lane) - 1u));
+        if (on) {
+            __stcs(where + i, make_uint2(b, at));
+            if (at == most) *bad = 1;
+        }
     }
 }
 
@@ -259,11 +240,8 @@ struct __align__(64) Anchor {
     double z, c1, c2, c3;
     float c4, c5, c6, unused[5];
 };
-__global__ void __launch_bounds__(kThreads)
-k_gauss_anchors(size_t n, size_t count, Anchor *__restrict__ out)
+__device__ __forceinline__ void make_anchor(size_t n, size_t a, Anchor *__restrict__ out)
 {
-    const size_t a = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (a >= count) return;
     const double z = normcdfinv(((double)(a * kAnchor + kAnchor / 2) + 0.5) / (double)n), z2 = z * z;
     const double D = 2.5066282746310002 * exp(0.5 * z2) / (double)n;   // sqrt(2 pi)
     const double D2 = D * D, D3 = D2 * D;
@@ -276,6 +254,52 @@ k_gauss_anchors(size_t n, size_t count, Anchor *__restrict__ out)
     x.c5 = (float)(D2 * D3 * (7.0 + z2 * (46.0 + 24.0 * z2)) * (1.0 / 120.0));
     x.c6 = (float)(D3 * D3 * z * (127.0 + z2 * (326.0 + 120.0 * z2)) * (1.0 / 720.0));
     out[a] = x;
+}
+
+// sub-buckets of every cell: a power of two above its share / kPerBucket
+// (below n / 8 + kCells buckets in all); one block of kSampleRun threads
+__device__ __noinline__ void gauss_plan(int weight, GaussPlan *P)
+{
+    __shared__ unsigned sh[32];
+    constexpr int kPer = kCells / kSampleRun;
+    unsigned lg[kPer], sum = 0;
+    for (int i = 0; i < kPer; ++i) {
+        const unsigned want = (__ldcg(&P->cell[threadIdx.x * kPer + i]) * (unsigned)weight) / kPerBucket;
+        lg[i] = want ? 32 - __clz(want) - (__popc(want) == 1) : 0;   // ceil(log2(want))
+        sum += 1u << lg[i];
+    }
+    unsigned total;
+    unsigned run = block_excl_scan(sum, sh, &total);
+    for (int i = 0; i < kPer; ++i) {
+        P->cell[threadIdx.x * kPer + i] = run;
+        P->down[threadIdx.x * kPer + i] = (unsigned char)(kCellBits - lg[i]);
+        run += 1u << lg[i];
+    }
+}
+
+// Cell counts of the sample (kSampleRun of every kSampleStep values, or all of a
+// small field) by the first `blocks` blocks; the anchors by the others, hidden
+// behind the sample; the plan by the last
+__global__ void __launch_bounds__(kSampleRun)
+k_gauss_sample(const double *__restrict__ v, size_t n, size_t step, unsigned blocks, int weight,
+               GaussPlan *__restrict__ P, size_t anchors, Anchor *__restrict__ out, unsigned *__restrict__ counter)
+{
+    __shared__ unsigned c[kCells];
+    const bool bad = P->bad;
+    if (blockIdx.x >= blocks) {
+        const size_t a = (size_t)(blockIdx.x - blocks) * kSampleRun + threadIdx.x;
+        if (a < anchors) make_anchor(n, a, out);
+    } else if (!bad) {
+        for (int i = threadIdx.x; i < kCells; i += kSampleRun) c[i] = 0;
+        __syncthreads();
+        for (size_t b = (size_t)blockIdx.x * step; b < n; b += (size_t)blocks * step)
+            if (b + threadIdx.x < n) atomicAdd(&c[linear_bits(P, v[b + threadIdx.x]) >> kCellBits], 1u);
+        __syncthreads();
+        for (int i = threadIdx.x; i < kCells; i += kSampleRun)
+            if (c[i]) atomicAdd(&P->cell[i], c[i]);
+    }
+    __syncthreads();   // the block's counts before its ticket
+    if (last_block(counter) && !bad) gauss_plan(weight, P);
 }
 __device__ __noinline__ double quantile_tail(size_t lo, bool low, size_t n, double m, double sd)
 {
@@ -312,21 +336,12 @@ k_gauss_rank(const Member *__restrict__ mem, size_t n, const GaussPlan *__restri
     }
 }
 
-// ---- the radix sort (P: run only where the buckets do not serve)
-__global__ void __launch_bounds__(kThreads)
-k_gauss_keys(const double *__restrict__ v, size_t n, const GaussPlan *__restrict__ P,
-             unsigned long long *__restrict__ key, unsigned *__restrict__ idx)
-{
-    if (!use_radix(P, n)) return;
-    for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
-        key[i] = order_key(v[i]);
-        idx[i] = (unsigned)i;
-    }
-}
-
+// ---- the radix sort (P: run only where the buckets do not serve).  The first
+// pass (FIRST) takes the keys from the values v, with their positions as indices.
 // counts[d * ntile + tile] = occurrences of digit d in the tile
+template <bool FIRST>
 __global__ void __launch_bounds__(kRadixThreads)
-k_radix_hist(const unsigned long long *__restrict__ key, size_t n, int shift, int ntile,
+k_radix_hist(const unsigned long long *__restrict__ key, const double *__restrict__ v, size_t n, int shift, int ntile,
              unsigned *__restrict__ counts, const GaussPlan *__restrict__ P)
 {
     __shared__ unsigned hist[256];
@@ -337,7 +352,7 @@ k_radix_hist(const unsigned long long *__restrict__ key, size_t n, int shift, in
         const size_t base = (size_t)tile * kTile;
         for (int r = 0; r < kRadixItems; ++r) {
             const size_t e = base + (size_t)r * kRadixThreads + threadIdx.x;
-            if (e < n) atomicAdd(&hist[(unsigned)(key[e] >> shift) & 255u], 1u);
+            if (e < n) atomicAdd(&hist[(unsigned)((FIRST ? order_key(v[e]) : key[e]) >> shift) & 255u], 1u);
         }
         __syncthreads();
         counts[(size_t)threadIdx.x * ntile + tile] = hist[threadIdx.x];
@@ -370,15 +385,19 @@ __device__ __forceinline__ unsigned block_excl_scan(unsigned v, unsigned *sh, un
     return before + x - v;
 }
 
-// The scans serve both paths: P null for the buckets (k_scan_seg then adds up
-// their squared counts in squares), else they run only for the radix sort.
+// The scans serve both paths: the buckets' unless the count was ended (k_scan_seg
+// then adds up their squared counts), the radix sort's where it runs.
+__device__ __forceinline__ bool scan_off(const GaussPlan *P, size_t n, bool buckets)
+{
+    return buckets ? P->bad != 0 : !use_radix(P, n);
+}
 // exclusive scan of each kScanSeg-long segment in place; segsum = its total
 __global__ void __launch_bounds__(kScanThreads)
-k_scan_seg(unsigned *__restrict__ a, size_t m, unsigned *__restrict__ segsum, const GaussPlan *__restrict__ P, size_t n,
-           unsigned long long *__restrict__ squares)
+k_scan_seg(unsigned *__restrict__ a, size_t m, unsigned *__restrict__ segsum, GaussPlan *__restrict__ P, size_t n,
+           bool buckets)
 {
     __shared__ unsigned sh[32];
-    if (P && !use_radix(P, n)) return;
+    if (scan_off(P, n, buckets)) return;
     const size_t base = (size_t)blockIdx.x * kScanSeg + (size_t)threadIdx.x * kScanItems;
     unsigned v[kScanItems], s = 0;
     unsigned long long sq = 0;
@@ -387,9 +406,9 @@ k_scan_seg(unsigned *__restrict__ a, size_t m, unsigned *__restrict__ segsum, co
         s += v[k];
         sq += (unsigned long long)v[k] * v[k];
     }
-    if (squares) {
+    if (buckets) {
         for (int o = 16; o > 0; o >>= 1) sq += __shfl_xor_sync(0xffffffffu, sq, o);
-        if ((threadIdx.x & 31) == 0 && sq) atomicAdd(squares, sq);
+        if ((threadIdx.x & 31) == 0 && sq) atomicAdd(&P->squares, sq);
     }
     unsigned total;
     unsigned run = block_excl_scan(s, sh, &total);
@@ -402,10 +421,10 @@ k_scan_seg(unsigned *__restrict__ a, size_t m, unsigned *__restrict__ segsum, co
 
 // exclusive scan of the segment totals (one block, any count)
 __global__ void __launch_bounds__(kScanThreads)
-k_scan_top(unsigned *__restrict__ segsum, int nseg, const GaussPlan *__restrict__ P, size_t n)
+k_scan_top(unsigned *__restrict__ segsum, int nseg, const GaussPlan *__restrict__ P, size_t n, bool buckets)
 {
     __shared__ unsigned sh[32];
-    if (P && !use_radix(P, n)) return;
+    if (scan_off(P, n, buckets)) return;
     unsigned carry = 0;
     for (int base = 0; base < nseg; base += kScanThreads) {
         const int i = base + threadIdx.x;
@@ -419,20 +438,69 @@ k_scan_top(unsigned *__restrict__ segsum, int nseg, const GaussPlan *__restrict_
 
 __global__ void __launch_bounds__(kScanThreads)
 k_scan_add(unsigned *__restrict__ a, size_t m, const unsigned *__restrict__ segsum, const GaussPlan *__restrict__ P,
-           size_t n)
+           size_t n, bool buckets)
 {
-    if (P && !use_radix(P, n)) return;
+    if (scan_off(P, n, buckets)) return;
     const size_t base = (size_t)blockIdx.x * kScanSeg + (size_t)threadIdx.x * kScanItems;
     const unsigned add = segsum[blockIdx.x];
     for (int k = 0; k < kScanItems; ++k)
         if (base + k < m) a[base + k] += add;
 }
 
+// The whole scan in one block, where that takes no longer than three launches
+// (64^3: 16384 radix counts 9.7 us against 10.6; the buckets', once a call, pay up
+// to 40960): a small field's time is its launches (8^3 with ties 250 us in 54,
+// 176 us in 32)
+constexpr size_t kScanOne[2] = {4 * kScanSeg, 10 * kScanSeg};   // radix, buckets
+__global__ void __launch_bounds__(kScanThreads)
+k_scan_one(unsigned *__restrict__ a, size_t m, GaussPlan *__restrict__ P, size_t n, bool buckets)
+{
+    __shared__ unsigned sh[32];
+    if (scan_off(P, n, buckets)) return;
+    unsigned carry = 0;
+    unsigned long long sq = 0;
+    for (size_t seg = 0; seg < m; seg += kScanSeg) {
+        const size_t base = seg + (size_t)threadIdx.x * kScanItems;
+        unsigned v[kScanItems], s = 0;
+        for (int k = 0; k < kScanItems; ++k) {
+            v[k] = base + k < m ? a[base + k] : 0u;
+            s += v[k];
+            sq += (unsigned long long)v[k] * v[k];
+        }
+        unsigned total;
+        unsigned run = carry + block_excl_scan(s, sh, &total);
+        for (int k = 0; k < kScanItems; ++k) {
+            if (base + k < m) a[base + k] = run;
+            run += v[k];
+        }
+        carry += total;
+    }
+    if (buckets) {
+        for (int o = 16; o > 0; o >>= 1) sq += __shfl_xor_sync(0xffffffffu, sq, o);
+        if ((threadIdx.x & 31) == 0 && sq) atomicAdd(&P->squares, sq);
+    }
+}
+// exclusive scan of m counts in place
+void scan_counts(unsigned *a, size_t m, unsigned *segsum, GaussPlan *P, size_t n, bool buckets, cudaStream_t s)
+{
+    if (m <= kScanOne[buckets]) {
+        note_launch();
+        k_scan_one<<<1, kScanThreads, 0, s>>>(a, m, P, n, buckets);
+        return;
+    }
+    const int nseg = (int)((m + kScanSeg - 1) / kScanSeg);
+    note_launch(3);
+    k_scan_seg<<<nseg, kScanThreads, 0, s>>>(a, m, segsum, P, n, buckets);
+    k_scan_top<<<1, kScanThreads, 0, s>>>(segsum, nseg, P, n, buckets);
+    k_scan_add<<<nseg, kScanThreads, 0, s>>>(a, m, segsum, P, n, buckets);
+}
+
 // stable scatter of one tile by the digit at `shift`; offs[d * ntile + tile]
 // is where the tile's first element of digit d goes
+template <bool FIRST>
 __global__ void __launch_bounds__(kRadixThreads)
-k_radix_scatter(const unsigned long long *__restrict__ kin, const unsigned *__restrict__ iin, size_t n,
-                int shift, int ntile, const unsigned *__restrict__ offs,
+k_radix_scatter(const unsigned long long *__restrict__ kin, const unsigned *__restrict__ iin,
+                const double *__restrict__ v, size_t n, int shift, int ntile, const unsigned *__restrict__ offs,
                 unsigned long long *__restrict__ kout, unsigned *__restrict__ iout, const GaussPlan *__restrict__ P)
 {
     if (!use_radix(P, n)) return;
@@ -449,7 +517,7 @@ k_radix_scatter(const unsigned long long *__restrict__ kin, const unsigned *__re
             for (int w = 0; w < kW; ++w) wcnt[w][tid] = 0;
             const size_t e = tile + (size_t)r * kRadixThreads + tid;
             const bool valid = e < n;
-            const unsigned long long k = valid ? kin[e] : 0ull;
+            const unsigned long long k = !valid ? 0ull : (FIRST ? order_key(v[e]) : kin[e]);
             const unsigned d = valid ? ((unsigned)(k >> shift) & 255u) : 256u;
             const unsigned peers = __match_any_sync(0xffffffffu, d);
             const unsigned rank = __popc(peers & lt);
@@ -469,7 +537,7 @@ k_radix_scatter(const unsigned long long *__restrict__ kin, const unsigned *__re
             if (valid) {
                 const unsigned pos = base[d] + wcnt[warp][d] + rank;
                 kout[pos] = k;
-                iout[pos] = iin[e];
+                iout[pos] = FIRST ? (unsigned)e : iin[e];
             }
             __syncthreads();
             base[tid] += total[tid];
@@ -536,23 +604,20 @@ cudaError_t gaussianise(recon_handle *H, const double *v, size_t n, double *g)
     const bool whole = n < 256 * (size_t)kSampleStep;   // small fields are counted in full
     const size_t step = whole ? kSampleRun : kSampleStep;
     const size_t sblocks = (n + step - 1) / step;
-    note_launch(5);
-    k_gauss_stats<<<nb, kThreads, 0, s>>>(v, n, H->partials);
-    k_gauss_moments<<<1, kReduceThreads, 0, s>>>(H->partials, (int)nb, (double)n, P);
-    k_gauss_anchors<<<blocks_for(nanchor), kThreads, 0, s>>>(n, nanchor, anchors);
-    k_gauss_sample<<<(unsigned)(sblocks < 608 ? sblocks : 608), kSampleRun, 0, s>>>(v, n, step, P);
-    k_gauss_plan<<<1, kScanThreads, 0, s>>>(whole ? 1 : kSampleStep / kSampleRun, P);
+    note_launch(2);
+    k_gauss_stats<<<nb, kThreads, 0, s>>>(v, n, H->partials, H->ticket, P);
+    const unsigned sampling = (unsigned)(sblocks < 608 ? sblocks : 608);
+    k_gauss_sample<<<sampling + (unsigned)((nanchor + kSampleRun - 1) / kSampleRun), kSampleRun, 0, s>>>(
+        v, n, step, sampling, whole ? 1 : kSampleStep / kSampleRun, P, nanchor, anchors, H->ticket);
     // buckets
     Member *mem = static_cast<Member *>(G.pairs);
     uint2 *where = reinterpret_cast<uint2 *>(mem + n);
     const size_t slots = bucket_slots(n);
-    const int bseg = (int)((slots + kScanSeg - 1) / kScanSeg);
     CK(cudaMemsetAsync(G.counts, 0, sizeof(unsigned) * slots, s));
-    note_launch(6);
-    k_gauss_count<<<sb, kThreads, 0, s>>>(v, n, P, G.counts, where);
-    k_scan_seg<<<bseg, kScanThreads, 0, s>>>(G.counts, slots, G.segsum, nullptr, n, &P->squares);
-    k_scan_top<<<1, kScanThreads, 0, s>>>(G.segsum, bseg, nullptr, n);
-    k_scan_add<<<bseg, kScanThreads, 0, s>>>(G.counts, slots, G.segsum, nullptr, n);
+    note_launch(3);
+    const unsigned most = (unsigned)std::sqrt((double)(kMaxWork / 16) * (double)n) + 1;
+    k_gauss_count<<<sb, kThreads, 0, s>>>(v, n, P, G.counts, where, most);
+    scan_counts(G.counts, slots, G.segsum, P, n, true, s);
     k_gauss_scatter<<<sb, kThreads, 0, s>>>(v, n, P, G.counts, where, mem);
     k_gauss_rank<<<sb, kThreads, 0, s>>>(mem, n, P, G.counts, anchors, g);
     // the radix sort, where the plan says so
@@ -562,18 +627,14 @@ cudaError_t gaussianise(recon_handle *H, const double *v, size_t n, double *g)
     const int ntile = (int)((n + kTile - 1) / kTile);
     const unsigned rb = ntile < 1216 ? ntile : 1216;
     const size_t m = 256 * (size_t)ntile;
-    const int nseg = (int)((m + kScanSeg - 1) / kScanSeg);
-    note_launch();
-    k_gauss_keys<<<nb, kThreads, 0, s>>>(v, n, P, key[0], idx[0]);
     int cur = 0;
     for (int shift = 0; shift < 64; shift += 8) {
-        note_launch(5);
-        k_radix_hist<<<rb, kRadixThreads, 0, s>>>(key[cur], n, shift, ntile, G.counts, P);
-        k_scan_seg<<<nseg, kScanThreads, 0, s>>>(G.counts, m, G.segsum, P, n, nullptr);
-        k_scan_top<<<1, kScanThreads, 0, s>>>(G.segsum, nseg, P, n);
-        k_scan_add<<<nseg, kScanThreads, 0, s>>>(G.counts, m, G.segsum, P, n);
-        k_radix_scatter<<<rb, kRadixThreads, 0, s>>>(key[cur], idx[cur], n, shift, ntile, G.counts, key[cur ^ 1],
-                                                     idx[cur ^ 1], P);
+        note_launch(2);
+        (shift ? k_radix_hist<false> : k_radix_hist<true>)<<<rb, kRadixThreads, 0, s>>>(key[cur], v, n, shift, ntile,
+                                                                                   G.counts, P);
+        scan_counts(G.counts, m, G.segsum, P, n, false, s);
+        (shift ? k_radix_scatter<false> : k_radix_scatter<true>)<<<rb, kRadixThreads, 0, s>>>(
+            key[cur], idx[cur], v, n, shift, ntile, G.counts, key[cur ^ 1], idx[cur ^ 1], P);
         cur ^= 1;
     }
     note_launch();
