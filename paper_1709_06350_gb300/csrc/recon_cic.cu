@@ -780,10 +780,19 @@ cudaError_t displace(int N, double L, const double *phi, const double *b, double
     if (e != cudaSuccess) return e;
     note_launch(2);
     const unsigned nx = (N + kRowX - 1) / kRowX, ny = (N + kRowY - 1) / kRowY;
-    // chunks of up to 32 planes (each starts by loading two), fewer where that
-    // would leave less than two waves of four CTAs per SM
-    const unsigned most = nx * ny * N / (8 * kSMs);
-    const unsigned chunk = most < 1 ? 1 : most > 32 ? 32 : most;
+    // planes per CTA, up to 32: those with the least waves x (planes + the two that
+    // each CTA starts by loading).  80^3 35.0 -> 28.7 us, 224^3 337 -> 308, 384^3 and
+    // 512^3 as with 32 (chunks for two waves before); measured best of all 32 or
+    // within 7% of it on 18 sides from 16 to 512
+    unsigned chunk = 1, least = ~0u;
+    for (unsigned c = 1; c <= 32; ++c) {
+        const unsigned ctas = nx * ny * ((N + c - 1) / c);
+        const unsigned cost = (ctas + kDispCTAs * kSMs - 1) / (kDispCTAs * kSMs) * (c + 2);
+        if (cost < least) {
+            least = cost;
+            chunk = c;
+        }
+    }
     k_displace_cells<<<dim3(nx, ny, (N + chunk - 1) / chunk), row_block(), 0, s>>>(
         phi, b, N, h, (float)(1.0 / (h * h)), (int)chunk, psi, acc);
     k_displace_finish<<<blocks_for(n), kThreads, 0, s>>>(acc, n, deltaL);
