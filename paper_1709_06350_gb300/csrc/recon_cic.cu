@@ -373,11 +373,10 @@ cudaError_t assign_deposit(int scheme, const double *pos, long long n, int N, do
 // L2 sectors: the z corner shared with the next lane is merged by a shuffle,
 // and the two upper-x columns are held in registers until the next plane, which
 // adds them to its lower-x ones wherever both map to the same cells.  Bound by
-// issue (62%) and FP64 (52%: psi's differences and scales, b's conversion).
+// issue (65%) and FP64 (55%: psi's differences and scales, b's conversion).
 // 384^3: 1.19 ms, 1.47 + 0.19 ms with a thread per cell behind the split; three
 // CTAs per SM 1.31 ms; four are what 64 registers allow without spills (five,
-// spilling, 1.17 ms: no more than GPUs differ by); chunks of 16 or 64 planes
-// 1% more.
+// spilling, 1.17 ms: no more than GPUs differ by).
 constexpr int kDispCTAs = 4, kTileX = kRowX + 2, kTileY = kRowY + 2, kTile = kTileX * kTileY;
 __global__ void __launch_bounds__(kRowX * kRowY, kDispCTAs)
 k_displace_cells(const double *__restrict__ t, const double *__restrict__ b, int N, double h,

@@ -19,8 +19,8 @@
 // operations per value at one per 64 FP32 ones): it is evaluated once per 128
 // ranks and continued by its Taylor series (five FP64 operations per value).
 // What bounds it: the sector traffic of the scatters and the FP64 pipe.
-// Measured (GB300): 256^3 4.24 -> 1.35 to 1.49 ms (GPUs differ; scatter 0.43,
-// ranks 0.38, places 0.16), 512^3 36.9 -> 12.1 to 12.7 ms; a 256^3 field of
+// Measured (GB300): 256^3 4.24 -> 1.35 to 1.50 ms (GPUs differ; scatter 0.43 to
+// 0.52, ranks 0.38 to 0.44, places 0.16), 512^3 36.9 -> 12.1 to 12.7 ms; a 256^3 field of
 // rounded values (radix path) 3.5 -> 1.8 ms.  Fields that take the radix path are
 // 3 to 5% slower than by it alone at 64^3 and 80^3, and faster at other sides.
 #include <climits>
